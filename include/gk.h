@@ -111,9 +111,11 @@ typedef struct gk_solver_s* gk_solver;
  * without a Time criterion run as ONE launch: a 16-CTA thread-block cluster
  * (the vectors the SpMVs read in distributed shared memory, the phases
  * separated by cluster barriers) up to 32,768 rows for GK_CG and 16,384 rows
- * for GK_BICGSTAB; and, for GK_CG from 32,769 to 262,144 rows when no row
- * has more than 64 entries, a cooperative grid of one CTA per SM (grid-wide
- * barriers in global memory).  check_every < 0 always takes the graph. */
+ * for GK_BICGSTAB; and, from 32,769 to 262,144 rows for GK_CG and to 1,024
+ * rows per SM (155,648 on 152 SMs) for GK_BICGSTAB, when no row has more than
+ * 64 entries and the vector entries a CTA's rows refer to fit its shared
+ * memory (not so for widely scattered columns), a cooperative grid of one CTA
+ * per SM (grid-wide reductions through global memory).  check_every < 0 always takes the graph. */
 typedef struct {
   int64_t max_iters;        /* GK_IR_CG: limit on the total of inner iterations      */
   double reduction_factor;
@@ -152,7 +154,8 @@ typedef struct {
 #define GK_FORM_HOST 1     /* iterations launched from the host (check_every > 0)      */
 #define GK_FORM_CLUSTER 2  /* one launch of a 16-CTA thread-block cluster (small CG  */
                            /* and BiCGSTAB)                                           */
-#define GK_FORM_GRID 3     /* one cooperative launch, grid-wide barriers (mid-size CG) */
+#define GK_FORM_GRID 3     /* one cooperative launch, grid-wide reductions (mid-size   */
+                           /* CG and BiCGSTAB)                                        */
 
 /* What a solver was built into. */
 typedef struct {

@@ -367,13 +367,17 @@ struct Solver {
   bool cl_stage = false;    // ... the CTA's rows of the matrix staged in shared memory
   int cl_nnz = 0;           // ... room for that many entries
   size_t cl_smem = 0;       // ... dynamic shared memory per CTA
-  int gr_grid = 0;          // GK_CG mid-size form: CTAs of the cooperative launch (0: not available)
+  int gr_grid = 0;          // GK_CG, GK_BICGSTAB mid-size form: CTAs of the cooperative launch (0: not available)
   int gr_rpt = 1, gr_rows = 0;
   bool gr_stage = false;            // its CTAs' rows of the matrix staged in shared memory
   int gr_nnz = 0;
   size_t gr_smem = 0;
-  double* gr_part = nullptr;        // its per-CTA partial sums
-  unsigned int* gr_sync = nullptr;  // its barrier words
+  int gr_halo_cap = 0;              // its largest halo
+  unsigned long long gr_epoch = 0;  // the next solve's sequence numbers start at gr_epoch << 40
+  ulonglong2* gr_words = nullptr;   // {value, sequence number}: the reductions', the abort word, the vectors'
+  int32_t* gr_halo_n = nullptr;     // halo entries of every CTA
+  int32_t* gr_halo_col = nullptr;   // and their columns
+  int32_t* gr_code = nullptr;       // per entry of the matrix, its column's place in the CTA's slice
 };
 
 // Mixed-precision iterative refinement (mixed.cu).
@@ -388,8 +392,9 @@ void ir_release(IrData* ir);
 int cluster_cg_plan(Solver* S);
 int cluster_cg_solve(Solver* S, cudaStream_t s);
 
-// CG of a mid-size system (32,769 .. 262,144 rows, rows of at most 64
-// entries) in one cooperative launch with grid-wide barriers (grid_cg.cu).
+// CG (32,769 .. 262,144 rows) and BiCGSTAB (from 32,769 rows to 1,024 per SM)
+// of a mid-size system with rows of at most 64 entries, in one cooperative
+// launch with grid-wide reductions (grid_cg.cu).
 int grid_cg_plan(Solver* S);
 int grid_cg_solve(Solver* S, cudaStream_t s);
 

@@ -511,8 +511,10 @@ void solver_release(Solver* S) {
   dfree(S->st);
   dfree(S->partials);
   dfree(S->counter);
-  dfree(S->gr_part);
-  dfree(S->gr_sync);
+  dfree(S->gr_words);
+  dfree(S->gr_halo_n);
+  dfree(S->gr_halo_col);
+  dfree(S->gr_code);
   if (S->h_st) cudaFreeHost(S->h_st);
   ir_release(S->ir);
   gmres_release(S->gm);
@@ -781,7 +783,7 @@ extern "C" int gk_solver_generate(gk_matrix hA, gk_precond hP, int32_t kind, con
     if (kind == GK_IR_CG && (rc = ir_generate(S))) break;
     if (kind == GK_GMRES && (rc = gmres_generate(S))) break;
     if ((kind == GK_CG || kind == GK_BICGSTAB) && (rc = cluster_cg_plan(S))) break;
-    if (kind == GK_CG && S->cl_lg < 0 && (rc = grid_cg_plan(S))) break;
+    if ((kind == GK_CG || kind == GK_BICGSTAB) && S->cl_lg < 0 && (rc = grid_cg_plan(S))) break;
   } while (false);
   if (prev != A->device) cudaSetDevice(prev);
   if (rc != GK_OK) return rc;
@@ -832,7 +834,7 @@ extern "C" int gk_solve(gk_solver h, const void* b, void* x, gk_status* status, 
       if ((rc = cluster_cg_solve(S, s))) break;
       if ((rc = enqueue_final(*S, s))) break;
       form = GK_FORM_CLUSTER;
-    } else if (S->kind == GK_CG && S->gr_grid > 0 && S->crit.check_every == 0 && !(S->crit.time_limit_s > 0)) {
+    } else if (S->gr_grid > 0 && S->crit.check_every == 0 && !(S->crit.time_limit_s > 0)) {
       // mid-size system: the whole iteration in one cooperative launch
       const gk_criteria& c = S->crit;
       solver_init_kernel<<<1, 1, 0, s>>>(S->st, c.reduction_factor, static_cast<long long>(c.max_iters), c.rel_to_b,
