@@ -218,7 +218,6 @@ struct Matrix {
   int32_t* rowptr = nullptr;
   int32_t* col = nullptr;
   double* val = nullptr;
-  std::vector<int32_t> h_rowptr;  // host copy of the row pointers (planning)
   // GK_CSR: rows sorted by decreasing length.  Rows of <= kSliceMaxLen
   // entries in slices of 32 rows, each slice column-major (entry k of lane l
   // at sl_off[c] + 32 k + l) and padded to its longest row with column -1;
@@ -273,7 +272,6 @@ struct Matrix {
   unsigned int* counter = nullptr;
   int* err = nullptr;
   SolverState* dot_st = nullptr;  // gk_apply_dot: receives the fused sum
-  int* h_flag = nullptr;          // pinned host words of the preconditioner generation's error check
   double* stage_in = nullptr;   // host-vector staging
   double* stage_out = nullptr;
   int max_grid = 0;             // partials hold max_grid * 2 doubles

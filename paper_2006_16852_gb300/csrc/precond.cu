@@ -63,7 +63,7 @@ __global__ void jacobi_scalar_kernel(const int32_t* __restrict__ rowptr, const i
     const bool found = at >= 0;
     if (found) d = __ldg(val + at);
     if (!found || d == 0.0) {
-      atomicMin(bad, r);
+      atomicMax(bad, INT_MAX - r);
       dinv[r] = 0.0;
     } else {
       dinv[r] = 1.0 / d;
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kBjRegThreads) bj_invert_kernel(int n, int bs,
           }
         }
       }
-      if (singular) atomicMin(bad, blk);
+      if (singular) atomicMax(bad, INT_MAX - blk);
       // inverse(i, orig[k]) = A[i][k]
 #pragma unroll
       for (int i = 0; i < BT; ++i)
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kBjWarps * 32) bj_generate_kernel(
       }
       __syncwarp();
     }
-    if (singular && i == 0) atomicMin(bad, blk);
+    if (singular && i == 0) atomicMax(bad, INT_MAX - blk);
     const int64_t off = static_cast<int64_t>(blk) * bs * bs;
     for (int e = i; e < m * m; e += GW) {  // row-major: e = ii * m + j
       const int ii = e / m, j = e - ii * m;
@@ -481,16 +481,9 @@ extern "C" int gk_precond_generate(gk_matrix h, int32_t block_size, void* stream
   P->bs = block_size;
   int rc = GK_OK;
   do {
-    // the error word: INT_MAX in, the smallest failing row or block out,
-    // through pinned host words (asynchronous copies, no staging)
-    if (!A->h_flag && cudaMallocHost(&A->h_flag, 2 * sizeof(int)) != cudaSuccess) {
-      A->h_flag = nullptr;
-      rc = cuda_error(cudaGetLastError(), "cudaMallocHost");
-      break;
-    }
-    A->h_flag[0] = INT_MAX;
-    if (cudaMemcpyAsync(A->err + 1, A->h_flag, sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess) {
-      rc = cuda_error(cudaGetLastError(), "cudaMemcpyAsync");
+    // the error word: 0, or INT_MAX - the smallest failing row or block
+    if (cudaMemsetAsync(A->err + 1, 0, sizeof(int), s) != cudaSuccess) {
+      rc = cuda_error(cudaGetLastError(), "cudaMemsetAsync");
       break;
     }
     if (block_size == 1) {
@@ -514,13 +507,14 @@ extern "C" int gk_precond_generate(gk_matrix h, int32_t block_size, void* stream
       rc = cuda_error(e, "Jacobi generate launch");
       break;
     }
-    if (cudaMemcpyAsync(A->h_flag + 1, A->err + 1, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    int word = 0;
+    if (cudaMemcpyAsync(&word, A->err + 1, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
       rc = cuda_error(cudaGetLastError(), "Jacobi generate");
       break;
     }
-    const int bad = A->h_flag[1];
-    if (bad != INT_MAX) {
+    if (word != 0) {
+      const int bad = INT_MAX - word;
       rc = block_size == 1 ? set_error(GK_ERR_SINGULAR, "zero or missing diagonal in row %d", bad)
                            : set_error(GK_ERR_SINGULAR, "diagonal block %d is singular", bad);
       break;
