@@ -32,7 +32,6 @@ namespace {
 constexpr int kLayers = 6;
 constexpr int kCh[kLayers + 1] = {2, 32, 32, 32, 32, 32, 1};
 constexpr int kConvThreads = 256;
-constexpr int kWgradRows = 4;  // image rows per weight-gradient block
 
 __device__ __forceinline__ float to_f(float v) { return v; }
 template <typename T>
@@ -105,97 +104,446 @@ __global__ void __launch_bounds__(kConvThreads) conv_fwd_kernel(const TI* __rest
   }
 }
 
-// Partial weight and bias gradients of one layer over kWgradRows image rows
-// of one sample:  dw[o, c, tap] += sum_x dy[b, o, y, x] x[b, c, y + d (ky-1), x + d (kx-1)],
-// dbias[o] += sum_x dy[b, o, y, x].  A thread owns CO_T output channels of one
-// input channel for one residue class of x (XSPLIT classes); the sums (slot
-// = block, STRIDE = COUT * CIN * 9 + COUT floats in the parameter layout)
-// of the block's residue classes are summed first (in class order, through
-// shared memory) and the block writes one slot; the slots are summed in a
-// fixed order by wgrad_chunk_kernel and wgrad_final_kernel.
-template <int CIN, int COUT>
-struct WgradShape {
-  static constexpr int CO_T = COUT >= 4 ? 4 : 1;
-  static constexpr int NG = CIN * (COUT / CO_T);
-  static constexpr int XSPLIT = kConvThreads / NG;
-  static constexpr int STRIDE = COUT * CIN * 9 + COUT;
-  static_assert(NG * XSPLIT == kConvThreads, "thread mapping");
-};
+// Two FP32 multiply-adds in one instruction, each rounded as fmaf.
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float v) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
 
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(kConvThreads) conv_wgrad_kernel(const float* __restrict__ x,
-                                                                  const float* __restrict__ dy, int H, int W,
-                                                                  int dil, float* __restrict__ partials) {
-  using S = WgradShape<CIN, COUT>;
-  extern __shared__ float sm[];
-  const int DS = W | 1;                  // odd row strides: conflict-free
-  const int XS = (W + 2 * dil) | 1;
-  float* dys = sm;                       // [COUT][DS]
-  float* xs = dys + COUT * DS;           // [3][CIN][XS], x position p stored at p + dil
+// The 32 -> 32 layers' convolution (forward and data gradient), as
+// conv_fwd_kernel sums it, bit for bit.  The FP32 pipe bounds it: 9,216
+// multiply-adds per pixel.  A 16-byte broadcast of shared memory holds its
+// pipe for 2 cycles and conv_fwd_kernel needs 8 per input value, which is
+// twice the time of the 32 multiply-adds; here a thread takes four pixels, so
+// each weight read serves four, and the multiply-adds go two output channels
+// to an instruction (the same rate, half the issue slots).  The four pixels
+// are d rows apart in one column, so they share input rows: 18 values per
+// input channel instead of 36, the next channel's loaded while this one's
+// are used.
+// Persistent blocks stage the weights once.  Measured (16 images of 256^2):
+// 440 - 460 us a layer against 700.
+constexpr int kC32Threads = 128;
+constexpr int kC32Ppt = 4;  // pixels per thread: rows y, y + d, y + 2 d, y + 3 d of one column
+// Columns per tile, and the (row class, four rows) units of a column.
+__host__ __device__ constexpr int c32_width(int W) { return W > 64 ? 128 : W > 32 ? 64 : 32; }
+__host__ __device__ constexpr int c32_units(int H, int dil) {
+  return dil * (((H + dil - 1) / dil + kC32Ppt - 1) / kC32Ppt);
+}
+constexpr size_t kC32Smem = sizeof(float) * (32 * 9 * 32 + 32);
+
+template <int MODE>
+__global__ void __launch_bounds__(kC32Threads, 2) conv32_kernel(const float* __restrict__ x,
+                                                                const float* __restrict__ w,
+                                                                const float* __restrict__ bias, int B, int H, int W,
+                                                                int dil, float* __restrict__ y,
+                                                                const float* __restrict__ mask) {
+  extern __shared__ __align__(16) float c32[];  // [c * 9 + tap][o], then the bias
+  float* const bs = c32 + 32 * 9 * 32;
   const int t = threadIdx.x;
-  const int g = t / S::XSPLIT, s = t - (t / S::XSPLIT) * S::XSPLIT;
-  const int ci = g / (COUT / S::CO_T), co0 = (g - ci * (COUT / S::CO_T)) * S::CO_T;
-  const int b = blockIdx.y;
-  const int y0 = blockIdx.x * kWgradRows;
-  const int HW = H * W;
-  float acc[S::CO_T][9], dacc[S::CO_T];
-#pragma unroll
-  for (int k = 0; k < S::CO_T; ++k) {
-    dacc[k] = 0.0f;
-#pragma unroll
-    for (int tp = 0; tp < 9; ++tp) acc[k][tp] = 0.0f;
+  for (int i = t; i < 32 * 9 * 32; i += kC32Threads) {
+    const int o = i / 288, ct = i - o * 288;  // coalesced reads
+    c32[ct * 32 + o] = w[i];
   }
-  for (int yy = y0; yy < min(y0 + kWgradRows, H); ++yy) {
-    __syncthreads();
-    for (int idx = t; idx < COUT * W; idx += kConvThreads) {
-      const int o = idx / W, xx = idx - o * W;
-      dys[o * DS + xx] = dy[(static_cast<int64_t>(b) * COUT + o) * HW + yy * W + xx];
+  if (t < 32) bs[t] = MODE != CONV_MASK ? bias[t] : 0.0f;
+  __syncthreads();
+  const int HW = H * W;
+  const int tw = c32_width(W), groups = kC32Threads / tw;
+  const int tiles_x = (W + tw - 1) / tw;
+  const int units = c32_units(H, dil), tiles_u = (units + groups - 1) / groups;
+  for (int item = blockIdx.x; item < tiles_x * tiles_u * B; item += gridDim.x) {
+    const int b = item / (tiles_x * tiles_u), r0 = item - b * (tiles_x * tiles_u);
+    const int ut = r0 / tiles_x, xt = r0 - ut * tiles_x;
+    const int unit = ut * groups + t / tw, j = xt * tw + t % tw;
+    const int y0 = unit % dil + kC32Ppt * dil * (unit / dil);  // the thread's first row
+    const bool mine = unit < units && j < W;
+    // which of the 6 x 3 inputs of the thread's pixels lie inside the image
+    unsigned int ok = 0u;
+#pragma unroll
+    for (int e = 0; e < 18; ++e) {
+      const int ii = y0 + dil * (e / 3 - 1), jj = j + dil * (e % 3 - 1);
+      if (mine && ii >= 0 && ii < H && jj >= 0 && jj < W) ok |= 1u << e;
     }
-    const int XW = W + 2 * dil;
-    for (int idx = t; idx < 3 * CIN * XW; idx += kConvThreads) {
-      const int row = idx / XW, q = idx - row * XW;
-      const int ky = row / CIN, c = row - ky * CIN;
-      const int iy = yy + dil * (ky - 1), ix = q - dil;
-      float v = 0.0f;
-      if (iy >= 0 && iy < H && ix >= 0 && ix < W) v = x[(static_cast<int64_t>(b) * CIN + c) * HW + iy * W + ix];
-      xs[row * XS + q] = v;
-    }
-    __syncthreads();
-    for (int xx = s; xx < W; xx += S::XSPLIT) {
-      float d[S::CO_T];
+    const int64_t at0 = static_cast<int64_t>(y0) * W + j;
+    const float* xc = x + static_cast<int64_t>(b) * 32 * HW;
+    float v[kC32Ppt + 2][3];
+    auto load = [&](const float* src, float (&dst)[kC32Ppt + 2][3]) {
 #pragma unroll
-      for (int k = 0; k < S::CO_T; ++k) d[k] = dys[(co0 + k) * DS + xx];
+      for (int e = 0; e < 18; ++e) {
+        dst[e / 3][e % 3] = 0.0f;
+        if ((ok >> e) & 1u) dst[e / 3][e % 3] = __ldg(src + at0 + dil * ((e / 3 - 1) * W + e % 3 - 1));
+      }
+    };
+    unsigned long long acc[kC32Ppt][16];
 #pragma unroll
-      for (int ky = 0; ky < 3; ++ky) {
-        const float* xr = xs + (ky * CIN + ci) * XS + xx;
+    for (int u = 0; u < kC32Ppt; ++u)
 #pragma unroll
-        for (int kx = 0; kx < 3; ++kx) {
-          const float v = xr[dil * kx];
+      for (int q = 0; q < 16; ++q) acc[u][q] = 0ull;
+    load(xc, v);
+#pragma unroll 1
+    for (int c = 0; c < 32; ++c) {
+      float nv[kC32Ppt + 2][3];
+      xc += HW;
+      if (c < 31) load(xc, nv);
 #pragma unroll
-          for (int k = 0; k < S::CO_T; ++k) acc[k][ky * 3 + kx] = fmaf(d[k], v, acc[k][ky * 3 + kx]);
+      for (int tap = 0; tap < 9; ++tap) {
+        const ulonglong2* wr = reinterpret_cast<const ulonglong2*>(c32 + (c * 9 + tap) * 32);
+        unsigned long long a[kC32Ppt];
+#pragma unroll
+        for (int u = 0; u < kC32Ppt; ++u) a[u] = dup2(v[u + tap / 3][tap % 3]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const ulonglong2 wv = wr[q];
+#pragma unroll
+          for (int u = 0; u < kC32Ppt; ++u) {
+            fma2(acc[u][2 * q], wv.x, a[u]);
+            fma2(acc[u][2 * q + 1], wv.y, a[u]);
+          }
         }
       }
-      if (ci == 0) {
 #pragma unroll
-        for (int k = 0; k < S::CO_T; ++k) dacc[k] += d[k];
+      for (int e = 0; e < 18; ++e) v[e / 3][e % 3] = nv[e / 3][e % 3];
+    }
+#pragma unroll
+    for (int u = 0; u < kC32Ppt; ++u) {
+      if (!mine || y0 + u * dil >= H) continue;
+      const int64_t ob = static_cast<int64_t>(b) * 32 * HW + at0 + static_cast<int64_t>(u * dil) * W;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const float2 r2 = unpack2(acc[u][q]);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int64_t at = ob + static_cast<int64_t>(2 * q + e) * HW;
+          float r = e ? r2.y : r2.x;
+          if (MODE == CONV_MASK) {
+            r = mask[at] > 0.0f ? r : 0.0f;
+          } else {
+            r += bs[2 * q + e];
+            if (MODE == CONV_RELU) r = fmaxf(r, 0.0f);
+          }
+          y[at] = r;
+        }
       }
     }
   }
-  __syncthreads();  // the staging area becomes the class reduction buffer
-  float* rs = sm + static_cast<int64_t>(s) * S::STRIDE;
+}
+
+// Asynchronous global -> shared copies of 4 or 16 bytes (cp.async, through
+// L1); the bytes past src_bytes are zero-filled, and with src_bytes 0 nothing
+// is read from src.
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, uint32_t src_bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
+               : "memory");
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t src_bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
+               : "memory");
+}
+// Waits for all of this thread's cp.async copies.
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Weight gradients, dw[o, c, tap] = sum_p dy[o, p] x[c, p + d tap], and bias
+// gradients sum_p dy[o, p], as partial sums: each block writes one slot of
+// COUT * CIN * 9 + COUT floats in the parameter layout, and
+// wgrad_chunk_kernel and wgrad_final_kernel add the slots in a fixed order.
+//
+// wgrad32_kernel (32 -> 32), bound by the FP32 pipe (9,216 multiply-adds per
+// pixel).  A work item is a strip of image rows y0, y0 + d, ... of one image
+// and one column segment; a thread owns 8 output channels x 1 input channel
+// x 9 taps for half of the segment's columns, so a column costs it 11 reads
+// of shared memory (two of 16 bytes) for 72 multiply-adds.  Consecutive rows of a strip share two of their
+// three input rows: a ring of four staged rows, filled by asynchronous copies
+// one row ahead, reads each input row once.  (One thread per 4 output
+// channels, 13 reads for 36 multiply-adds and all three input rows staged
+// again for every row took 1,600 us a layer on 16 images of 256^2; this form
+// 555, and 740 at dilation 64.)
+constexpr int kW32Threads = 256;
+constexpr int kW32Dy = 36;  // floats per staged column of dy: 32, padded so that the transposing copies spread over the banks
+constexpr int kW32Stride = 32 * 32 * 9 + 32;
+
+// Columns per segment: narrower at wide dilations, whose staged rows are
+// mostly halo, so that two blocks fit an SM.
+__host__ __device__ constexpr int w32_seg(int dil) { return dil > 32 ? 32 : 64; }
+__host__ __device__ constexpr int w32_xs(int dil) { return (w32_seg(dil) + 2 * dil) | 1; }  // floats per staged row of x: odd
+__host__ __device__ constexpr size_t w32_smem(int dil) {
+  const size_t stage = 4 * 32 * static_cast<size_t>(w32_xs(dil)) + 2 * static_cast<size_t>(w32_seg(dil)) * kW32Dy;
+  return sizeof(float) * (stage > kW32Stride ? stage : kW32Stride);
+}
+
+// A thread's sums go to the block's slot after this many products, so that
+// no sum is longer than before the slots (kWgradRows * W was 1,024).
+constexpr int kW32Run = 512;
+
+// Rows per strip: at most 16, and few enough that every resident block gets
+// about six items (a strip stages two rows more than it multiplies).
+int w32_rows(int B, int H, int W, int dil) {
+  const int64_t columns = static_cast<int64_t>(B) * ((W + w32_seg(dil) - 1) / w32_seg(dil));
+  const int64_t want = 6 * 2 * static_cast<int64_t>(sm_count());
+  const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(16, columns * H / want));
+  return static_cast<int>(std::min<int64_t>(rows, (H + dil - 1) / dil));
+}
+int64_t w32_items(int B, int H, int W, int dil) {
+  const int rows = w32_rows(B, H, W, dil), per_class = (H + dil - 1) / dil;
+  return static_cast<int64_t>(B) * ((W + w32_seg(dil) - 1) / w32_seg(dil)) * dil * ((per_class + rows - 1) / rows);
+}
+
+__global__ void __launch_bounds__(kW32Threads, 2) wgrad32_kernel(const float* __restrict__ x,
+                                                                 const float* __restrict__ dy, int B, int H, int W,
+                                                                 int dil, int rows, float* __restrict__ partials) {
+  extern __shared__ __align__(16) float w32[];
+  const int seg = w32_seg(dil), XS = w32_xs(dil);
+  float* const dys = w32;                          // [2][seg][kW32Dy]
+  float* const xs = w32 + 2 * seg * kW32Dy;        // [4][32][XS], column x0 + j at j + dil
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int co0 = 8 * (lane & 3), ci = (lane >> 2) + 8 * (warp & 3), half = warp >> 2;
+  const int warp_u = __shfl_sync(0xffffffffu, warp & 3, 0);  // uniform: 0 sums the bias gradient
+  const int HW = H * W;
+  const int tiles_x = (W + seg - 1) / seg;
+  const int per_class = (H + dil - 1) / dil, chunks = (per_class + rows - 1) / rows;
+  const int n_items = B * tiles_x * dil * chunks;
+  float acc[9][8], dacc[8];
 #pragma unroll
-  for (int k = 0; k < S::CO_T; ++k) {
+  for (int k = 0; k < 8; ++k) {
+    dacc[k] = 0.0f;
 #pragma unroll
-    for (int tp = 0; tp < 9; ++tp) rs[((co0 + k) * CIN + ci) * 9 + tp] = acc[k][tp];
-    if (ci == 0) rs[COUT * CIN * 9 + co0 + k] = dacc[k];
+    for (int tap = 0; tap < 9; ++tap) acc[tap][k] = 0.0f;
   }
-  __syncthreads();
-  float* out = partials + (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * S::STRIDE;
-  for (int e = t; e < S::STRIDE; e += kConvThreads) {
-    float sum = 0.0f;
+  int run = 0;         // products in each of the thread's sums
+  bool stored = false;  // the block's slot holds earlier sums
+  float* const out = partials + static_cast<int64_t>(blockIdx.x) * kW32Stride;
+  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    int rest = item;
+    const int ch = rest % chunks;
+    rest /= chunks;
+    const int cls = rest % dil;
+    rest /= dil;
+    const int xt = rest % tiles_x;
+    const int b = rest / tiles_x;
+    const int x0 = xt * seg, y0 = cls + ch * rows * dil;
+    const int nrow = y0 < H ? min(rows, (H - 1 - y0) / dil + 1) : 0;
+    const float* xb = x + static_cast<int64_t>(b) * 32 * HW;
+    const float* db = dy + static_cast<int64_t>(b) * 32 * HW;
+    const int xw = seg + 2 * dil;
+    // input row yy (zeros outside the image) into ring slot q: a warp takes
+    // a channel at a time
+    auto stage_x = [&](int yy, int q) {
+      for (int c = warp; c < 32; c += kW32Threads / 32) {
+        float* dst = xs + (q * 32 + c) * XS;
+        const float* src = xb + static_cast<int64_t>(c) * HW + static_cast<int64_t>(yy) * W;
+        for (int j = lane; j < xw; j += 32) {
+          const int xx = x0 - dil + j;
+          const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
+          cp_async4(dst + j, in ? src + xx : x, in ? 4u : 0u);
+        }
+      }
+    };
+    // output-gradient row yy, transposed: 8 columns x 4 channels per warp
+    // and copy, which read whole sectors and write 32 different banks
+    auto stage_dy = [&](int yy, int q) {
+      float* dst = dys + q * seg * kW32Dy;
+      for (int e = warp; e < seg; e += kW32Threads / 32) {  // seg / 8 column groups x 8 channel groups
+        const int j = (e >> 3) * 8 + (lane >> 2), c = (e & 7) * 4 + (lane & 3);
+        const bool in = x0 + j < W;
+        cp_async4(dst + j * kW32Dy + c, in ? db + static_cast<int64_t>(c) * HW + static_cast<int64_t>(yy) * W + x0 + j : dy,
+                  in ? 4u : 0u);
+      }
+    };
+    __syncthreads();  // the previous item's rows (and sums) have been read
+    if (nrow > 0) {
+      stage_x(y0 - dil, 0);
+      stage_x(y0, 1);
+      stage_x(y0 + dil, 2);
+      stage_dy(y0, 0);
+    }
+    for (int k = 0; k < nrow; ++k) {
+      cp_async_wait_all();
+      __syncthreads();
+      if (k + 1 < nrow) {  // the slots of input row k - 2 and of dy row k - 1: every warp is past them
+        stage_x(y0 + (k + 2) * dil, (k + 3) & 3);
+        stage_dy(y0 + (k + 1) * dil, (k + 1) & 1);
+      }
+      const float* dr = dys + (k & 1) * seg * kW32Dy + co0;
+      const float* xr[3];
 #pragma unroll
-    for (int c = 0; c < S::XSPLIT; ++c) sum += sm[c * S::STRIDE + e];
-    out[e] = sum;
+      for (int ky = 0; ky < 3; ++ky) xr[ky] = xs + (((k + ky) & 3) * 32 + ci) * XS;
+      const int j0 = half * (seg / 2);
+#pragma unroll 2
+      for (int j = j0; j < j0 + seg / 2; ++j) {
+        const float4 d0 = *reinterpret_cast<const float4*>(dr + j * kW32Dy);
+        const float4 d1 = *reinterpret_cast<const float4*>(dr + j * kW32Dy + 4);
+        const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+        for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+          for (int kx = 0; kx < 3; ++kx) {
+            const float v = xr[ky][j + dil * kx];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[ky * 3 + kx][k] = fmaf(d[k], v, acc[ky * 3 + kx][k]);
+          }
+        if (warp_u == 0) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) dacc[k] += d[k];
+        }
+      }
+    }
+    run += nrow * (seg / 2);
+    if (run < kW32Run && item + static_cast<int>(gridDim.x) < n_items) continue;
+    // the halves' sums meet in the staging area, then go to the block's slot
+    __syncthreads();
+#pragma unroll
+    for (int h = 1; h >= 0; --h) {
+      if (half == h) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+#pragma unroll
+          for (int tap = 0; tap < 9; ++tap) {
+            const int e = ((co0 + k) * 32 + ci) * 9 + tap;
+            w32[e] = h ? acc[tap][k] : w32[e] + acc[tap][k];
+            acc[tap][k] = 0.0f;
+          }
+          if (ci == 0) {
+            const int e = 32 * 32 * 9 + co0 + k;
+            w32[e] = h ? dacc[k] : w32[e] + dacc[k];
+          }
+          dacc[k] = 0.0f;
+        }
+      }
+      __syncthreads();
+    }
+    for (int e = t; e < kW32Stride; e += kW32Threads) out[e] = stored ? out[e] + w32[e] : w32[e];
+    stored = true;
+    run = 0;
+  }
+}
+
+// wgrad_thin_kernel: the layers with a thin side (2 -> 32 and 32 -> 1), bound
+// by reading the 32-channel tensor (dy, or x) once.  A lane takes a column, a
+// warp 4 of the 32 channels.  For the 2 -> 32 layer the wide tensor is dy and
+// the thin one x, read at p + d tap; for the 32 -> 1 layer the wide one is x,
+// and x[q] meets dy at q - d tap.  A block takes kThinRows rows y0, y0 + d,
+// ..., so that a row adds 3 thin values per channel to the 6 kept from the
+// rows before; the next row's values are loaded while this one's are used.
+// At the end the lanes are added by a butterfly.  (16 images of 256^2:
+// 116 and 83 us, against 217 and 337 with both tensors staged in
+// shared memory, one thread per channel pair; reading all 9 thin values of
+// every pixel took 181 and 143.)
+constexpr int kThinRows = 8;
+
+// Blocks per image: (row class, kThinRows rows) units.
+__host__ __device__ constexpr int thin_units(int H, int dil) {
+  return dil * (((H + dil - 1) / dil + kThinRows - 1) / kThinRows);
+}
+
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(256, 2) wgrad_thin_kernel(const float* __restrict__ x,
+                                                            const float* __restrict__ dy, int H, int W, int dil,
+                                                            float* __restrict__ partials) {
+  static_assert((CIN == 32) != (COUT == 32), "one wide side");
+  constexpr bool kWideOut = COUT == 32;
+  constexpr int T = kWideOut ? CIN : COUT;  // thin channels
+  constexpr int STRIDE = COUT * CIN * 9 + COUT;
+  const int lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x) >> 5, 0);  // uniform
+  const int b = blockIdx.y, unit = blockIdx.x;
+  const int y0 = unit % dil + kThinRows * dil * (unit / dil);
+  const int nrow = y0 < H ? min(kThinRows, (H - 1 - y0) / dil + 1) : 0;
+  const int HW = H * W;
+  const float* wide = (kWideOut ? dy : x) + (static_cast<int64_t>(b) * 32 + 4 * warp) * HW;
+  const float* thin = (kWideOut ? x : dy) + static_cast<int64_t>(b) * T * HW;
+  float acc[4][T][9], sum[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    sum[k] = 0.0f;
+#pragma unroll
+    for (int c = 0; c < T; ++c)
+#pragma unroll
+      for (int tap = 0; tap < 9; ++tap) acc[k][c][tap] = 0.0f;
+  }
+  for (int x0 = 0; x0 < W; x0 += 32) {
+    const int xx = x0 + lane;
+    auto load_thin = [&](int m, float (&dst)[T][3]) {  // row m of the unit, columns xx - d, xx, xx + d
+      const int ii = y0 + m * dil;
+#pragma unroll
+      for (int c = 0; c < T; ++c)
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          const int jj = xx + dil * (e - 1);
+          dst[c][e] = 0.0f;
+          if (ii >= 0 && ii < H && jj >= 0 && jj < W)
+            dst[c][e] = __ldg(thin + static_cast<int64_t>(c) * HW + static_cast<int64_t>(ii) * W + jj);
+        }
+    };
+    auto load_wide = [&](int m, float (&dst)[4]) {
+      const int ii = y0 + m * dil;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        dst[k] = 0.0f;
+        if (m < nrow && xx < W)
+          dst[k] = __ldg(wide + static_cast<int64_t>(k) * HW + static_cast<int64_t>(ii) * W + xx);
+      }
+    };
+    float v[3][T][3], nv[T][3], a[4], na[4];  // v: thin rows m - 1, m, m + 1
+    load_thin(-1, v[1]);
+    load_thin(0, v[2]);
+    load_thin(1, nv);
+    load_wide(0, na);
+#pragma unroll 1
+    for (int m = 0; m < nrow; ++m) {
+#pragma unroll
+      for (int c = 0; c < T; ++c)
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          v[0][c][e] = v[1][c][e];
+          v[1][c][e] = v[2][c][e];
+          v[2][c][e] = nv[c][e];
+        }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) a[k] = na[k];
+      load_thin(m + 2, nv);
+      load_wide(m + 1, na);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int c = 0; c < T; ++c)
+#pragma unroll
+          for (int tap = 0; tap < 9; ++tap) {
+            const int e = kWideOut ? tap : 8 - tap;
+            acc[k][c][tap] = fmaf(a[k], v[e / 3][c][e % 3], acc[k][c][tap]);
+          }
+      if (kWideOut) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) sum[k] += a[k];
+      } else if (xx < W) {
+        sum[0] += v[1][0][1];  // dy itself
+      }
+    }
+  }
+  float* out = partials + (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * STRIDE;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int w = 4 * warp + k;  // the wide channel
+#pragma unroll
+    for (int c = 0; c < T; ++c)
+#pragma unroll
+      for (int tap = 0; tap < 9; ++tap) {
+        float r[1] = {acc[k][c][tap]};
+        warp_sum<1, float>(r);
+        if (lane == 0) out[(kWideOut ? w * CIN + c : w) * 9 + tap] = r[0];
+      }
+    if (kWideOut || (warp == 0 && k == 0)) {
+      float r[1] = {sum[k]};
+      warp_sum<1, float>(r);
+      if (lane == 0) out[COUT * CIN * 9 + (kWideOut ? w : 0)] = r[0];
+    }
   }
 }
 
@@ -410,16 +758,6 @@ constexpr int kTcMaxDil = 64;                   // largest dilation (gk_wsnet_cr
 constexpr uint32_t kTcChunkB = 32 * 16;         // bytes between 8-channel chunks of a tap's weights
 constexpr int kTcPacked = 9 * 4 * 32 * 8;       // packed BF16 weights of one 32 -> 32 layer
 constexpr int kTcMidLayers = kLayers - 2;
-
-// 16-byte asynchronous global -> shared copy through L1 (cp.async); the
-// bytes past src_bytes (0 or 16) are zero-filled, and with src_bytes 0
-// nothing is read from src.
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
-               : "memory");
-}
-// Waits for all of this thread's cp.async copies.
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Shared memory of a block: this header, then the ring of three staged
 // input rows, [row slot][chunk][pixel slot][8 channels], win = 128 + 2 dil
@@ -879,15 +1217,28 @@ int launch_conv(const TI* x, const TW* w, const TW* bias, int B, int H, int W, i
   return GK_OK;
 }
 
-template <typename TI, typename TW, typename TO>
-int forward_layer(int l, const TI* x, const TW* w, const TW* bias, int B, int H, int W, int dil, TO* y,
+template <int MODE>
+int launch_conv32(const float* x, const float* w, const float* bias, int B, int H, int W, int dil, float* y,
+                  const float* mask, cudaStream_t s) {
+  const int tw = c32_width(W), groups = kC32Threads / tw;
+  const int64_t items =
+      static_cast<int64_t>(B) * ((W + tw - 1) / tw) * ((c32_units(H, dil) + groups - 1) / groups);
+  const int grid = static_cast<int>(std::min<int64_t>(items, 2 * static_cast<int64_t>(sm_count())));
+  conv32_kernel<MODE><<<grid, kC32Threads, kC32Smem, s>>>(x, w, bias, B, H, W, dil, y, mask);
+  GK_TRY_CUDA(cudaGetLastError());
+  return GK_OK;
+}
+
+int forward_layer(int l, const float* x, const float* w, const float* bias, int B, int H, int W, int dil, float* y,
                   cudaStream_t s) {
   if (l == 0) return launch_conv<2, 32, CONV_RELU>(x, w, bias, B, H, W, dil, y, nullptr, s);
-  if (l < kLayers - 1) return launch_conv<32, 32, CONV_RELU>(x, w, bias, B, H, W, dil, y, nullptr, s);
+  if (l < kLayers - 1) return launch_conv32<CONV_RELU>(x, w, bias, B, H, W, dil, y, nullptr, s);
   return launch_conv<32, 1, CONV_LINEAR>(x, w, bias, B, H, W, dil, y, nullptr, s);
 }
 
-size_t wgrad_smem(int cin, int cout, int W, int dil) {
+// The documented limit on the width: the shared memory that one row of a
+// layer's two tensors, three input rows with their halo, would take.
+size_t width_limit_bytes(int cin, int cout, int W, int dil) {
   const int co_t = cout >= 4 ? 4 : 1;
   const size_t xsplit = kConvThreads / (cin * (cout / co_t));
   const size_t staging = static_cast<size_t>(cout) * (W | 1) + 3 * static_cast<size_t>(cin) * ((W + 2 * dil) | 1);
@@ -895,21 +1246,30 @@ size_t wgrad_smem(int cin, int cout, int W, int dil) {
   return sizeof(float) * std::max(staging, classes);
 }
 
+// Slots of a layer's weight-gradient partials for a batch of B.
+int64_t wgrad_slots(int cin, int cout, int B, int H, int W, int dil) {
+  if (cin == 32 && cout == 32) return std::min<int64_t>(w32_items(B, H, W, dil), 2 * sm_count());
+  return static_cast<int64_t>(B) * thin_units(H, dil);
+}
+
 template <int CIN, int COUT>
 int launch_wgrad(const WsNet& N, const float* x, const float* dy, int B, int dil, float* grads, cudaStream_t s) {
-  using S = WgradShape<CIN, COUT>;
-  const size_t smem = wgrad_smem(CIN, COUT, N.W, dil);
-  GK_TRY(set_smem(conv_wgrad_kernel<CIN, COUT>, smem));
-  const dim3 grid((N.H + kWgradRows - 1) / kWgradRows, B);
-  const int64_t nslots = static_cast<int64_t>(grid.x) * grid.y;
-  if (nslots * S::STRIDE > N.partial_floats) return set_error(GK_ERR_UNSUPPORTED, "wsnet: gradient scratch too small");
-  conv_wgrad_kernel<CIN, COUT><<<grid, kConvThreads, smem, s>>>(x, dy, N.H, N.W, dil, N.partials);
+  constexpr int STRIDE = COUT * CIN * 9 + COUT;
+  const int64_t nslots = wgrad_slots(CIN, COUT, B, N.H, N.W, dil);
+  if (nslots * STRIDE > N.partial_floats) return set_error(GK_ERR_UNSUPPORTED, "wsnet: gradient scratch too small");
+  if constexpr (CIN == 32 && COUT == 32) {
+    wgrad32_kernel<<<static_cast<int>(nslots), kW32Threads, w32_smem(dil), s>>>(
+        x, dy, B, N.H, N.W, dil, w32_rows(B, N.H, N.W, dil), N.partials);
+  } else {
+    wgrad_thin_kernel<CIN, COUT>
+        <<<dim3(thin_units(N.H, dil), B), 256, 0, s>>>(x, dy, N.H, N.W, dil, N.partials);
+  }
   GK_TRY_CUDA(cudaGetLastError());
   const int nch = static_cast<int>(std::min<int64_t>(kReduceChunks, nslots));
   const int64_t per = (nslots + nch - 1) / nch;
-  wgrad_chunk_kernel<<<dim3((S::STRIDE + 255) / 256, nch), 256, 0, s>>>(N.partials, nslots, S::STRIDE, per, N.chunk);
+  wgrad_chunk_kernel<<<dim3((STRIDE + 255) / 256, nch), 256, 0, s>>>(N.partials, nslots, STRIDE, per, N.chunk);
   GK_TRY_CUDA(cudaGetLastError());
-  wgrad_final_kernel<<<(S::STRIDE + 255) / 256, 256, 0, s>>>(N.chunk, nch, S::STRIDE, grads);
+  wgrad_final_kernel<<<(STRIDE + 255) / 256, 256, 0, s>>>(N.chunk, nch, STRIDE, grads);
   GK_TRY_CUDA(cudaGetLastError());
   return GK_OK;
 }
@@ -924,8 +1284,7 @@ int check_batch(const WsNet* N, int32_t B) {
 int forward_f32(WsNet& N, int B, const float* x, cudaStream_t s) {
   const float* in = x;
   for (int l = 0; l < kLayers; ++l) {
-    GK_TRY((forward_layer<float, float, float>(l, in, N.p + N.off_w[l], N.p + N.off_b[l], B, N.H, N.W, N.dil[l],
-                                               N.act[l + 1], s)));
+    GK_TRY(forward_layer(l, in, N.p + N.off_w[l], N.p + N.off_b[l], B, N.H, N.W, N.dil[l], N.act[l + 1], s));
     in = N.act[l + 1];
   }
   return GK_OK;
@@ -962,8 +1321,8 @@ int gradients(WsNet& N, int B, const float* x, const float* target, cudaStream_t
       GK_TRY((launch_conv<1, 32, CONV_MASK, float, float, float>(gcur, N.wflip + N.off_w[l], nullptr, B, N.H, N.W,
                                                                  N.dil[l], gnext, N.act[l], s)));
     else
-      GK_TRY((launch_conv<32, 32, CONV_MASK, float, float, float>(gcur, N.wflip + N.off_w[l], nullptr, B, N.H,
-                                                                  N.W, N.dil[l], gnext, N.act[l], s)));
+      GK_TRY(launch_conv32<CONV_MASK>(gcur, N.wflip + N.off_w[l], nullptr, B, N.H, N.W, N.dil[l], gnext, N.act[l],
+                                      s));
     gcur = gnext;
     pp = 1 - pp;
   }
@@ -1058,7 +1417,7 @@ extern "C" int gk_wsnet_create(int32_t H, int32_t W, int32_t batch_max, const in
   int smem_max = 0;
   GK_TRY_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, N->device));
   for (int l = 0; l < kLayers; ++l)
-    if (wgrad_smem(kCh[l], kCh[l + 1], W, N->dil[l]) > static_cast<size_t>(smem_max))
+    if (width_limit_bytes(kCh[l], kCh[l + 1], W, N->dil[l]) > static_cast<size_t>(smem_max))
       return set_error(GK_ERR_UNSUPPORTED, "gk_wsnet_create: width %d with dilation %d needs too much shared memory",
                        W, N->dil[l]);
   int64_t* by = &N->device_bytes;
@@ -1076,21 +1435,25 @@ extern "C" int gk_wsnet_create(int32_t H, int32_t W, int32_t batch_max, const in
   GK_TRY(dalloc_n(&N->wtc, static_cast<size_t>(kTcMidLayers) * kTcPacked, by));
   GK_TRY(dalloc_n(&N->err, 1, by));
   GK_TRY_CUDA(cudaMemset(N->err, 0, sizeof(int)));
+  // (process-wide attributes: the most any network's dilations need)
+  GK_TRY(set_smem(wgrad32_kernel, std::max(w32_smem(kTcMaxDil), w32_smem(32))));
+  GK_TRY(set_smem(conv32_kernel<CONV_RELU>, kC32Smem));
+  GK_TRY(set_smem(conv32_kernel<CONV_MASK>, kC32Smem));
   GK_TRY(set_smem(conv_tc_kernel<false>, tc_smem_bytes(kTcMaxDil)));
   GK_TRY(set_smem(conv_tc_kernel<true>, tc_smem_bytes(kTcMaxDil) + kTcLastBytes));
   // the grid of each layer is sized from its shared-memory footprint (the
   // occupancy query has been seen to report 1 for this kernel where 3 fit)
   GK_TRY_CUDA(cudaDeviceGetAttribute(&N->tc_smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, N->device));
   GK_TRY_CUDA(cudaDeviceGetAttribute(&N->tc_reserved, cudaDevAttrReservedSharedMemoryPerBlock, N->device));
-  // weight-gradient slots: the largest layer's count
+  // weight-gradient slots: the most any layer and batch needs
   int64_t pf = 0;
-  const int64_t blocks = static_cast<int64_t>((H + kWgradRows - 1) / kWgradRows) * batch_max;
-  pf = std::max<int64_t>(pf, blocks * WgradShape<2, 32>::STRIDE);
-  pf = std::max<int64_t>(pf, blocks * WgradShape<32, 32>::STRIDE);
-  pf = std::max<int64_t>(pf, blocks * WgradShape<32, 1>::STRIDE);
+  for (int l = 0; l < kLayers; ++l)
+    for (int B = 1; B <= batch_max; ++B)
+      pf = std::max(pf, wgrad_slots(kCh[l], kCh[l + 1], B, H, W, N->dil[l]) *
+                            (static_cast<int64_t>(kCh[l]) * kCh[l + 1] * 9 + kCh[l + 1]));
   N->partial_floats = pf;
   GK_TRY(dalloc_n(&N->partials, static_cast<size_t>(pf), by));
-  GK_TRY(dalloc_n(&N->chunk, static_cast<size_t>(kReduceChunks) * WgradShape<32, 32>::STRIDE, by));
+  GK_TRY(dalloc_n(&N->chunk, static_cast<size_t>(kReduceChunks) * kW32Stride, by));
   const int rg = 8 * sm_count() + 8;
   GK_TRY(dalloc_n(&N->red, static_cast<size_t>(rg + 4), by));
   GK_TRY(dalloc_n(&N->counter, 1, by));
