@@ -236,18 +236,14 @@ __global__ void __launch_bounds__(kC32Threads, 2) conv32_kernel(const float* __r
   }
 }
 
-// Asynchronous global -> shared copies of 4 or 16 bytes (cp.async, through
-// L1); the bytes past src_bytes are zero-filled, and with src_bytes 0 nothing
-// is read from src.
+// Asynchronous global -> shared copy of 4 bytes (cp.async, through L1); the
+// bytes past src_bytes are zero-filled, and with src_bytes 0 nothing is read
+// from src.
 __device__ __forceinline__ void cp_async4(void* dst, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
                : "memory");
 }
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(src_bytes)
-               : "memory");
-}
 // Waits for all of this thread's cp.async copies.
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -751,7 +747,8 @@ __global__ void scale_kernel(double* __restrict__ x0, const double* __restrict__
 // worth the name and runs on the CUDA cores, reading NHWC.
 // ---------------------------------------------------------------------------
 
-constexpr int kTcThreads = 128;                 // 4 warps: one TMEM lane quarter each
+constexpr int kTcThreads = 192;                 // 4 epilogue warps (one TMEM lane quarter each), an MMA warp, a copy warp
+constexpr int kTcFirstThreads = 128;
 constexpr int kTcTile = 128;                    // pixels per tile (MMA M)
 constexpr int kTcStripMax = 16;                 // output rows per work item (a strip), at most
 constexpr int kTcMaxDil = 64;                   // largest dilation (gk_wsnet_create checks it)
@@ -759,18 +756,30 @@ constexpr uint32_t kTcChunkB = 32 * 16;         // bytes between 8-channel chunk
 constexpr int kTcPacked = 9 * 4 * 32 * 8;       // packed BF16 weights of one 32 -> 32 layer
 constexpr int kTcMidLayers = kLayers - 2;
 
-// Shared memory of a block: this header, then the ring of three staged
-// input rows, [row slot][chunk][pixel slot][8 channels], win = 128 + 2 dil
-// pixel slots per chunk: sized per layer, so that layers of small dilation
-// fit more blocks per SM.
+// Activations between layers: per image row, four planes (8-channel chunks)
+// of W pixels x 16 bytes, so that a window of a row is four contiguous runs
+// for the bulk copies and a warp's epilogue stores are contiguous.
+__device__ __forceinline__ int64_t tc_act(int64_t row, int chunk, int W, int px) {  // in 16-byte units
+  return (row * 4 + chunk) * W + px;
+}
+
+// Shared memory of a block: this header, then the ring of kTcRing staged
+// input rows, [row slot][chunk][pixel slot][8 channels], 128 + 2 dil pixel
+// slots per chunk.
+constexpr int kTcRing = 5;
 struct TcSmem {
   __nv_bfloat16 b[kTcPacked];           // [tap][chunk][out][8 channels]
   float bias[32];
-  uint64_t bar;
+  uint64_t full[kTcRing];               // a slot's row has landed
+  uint64_t free_[kTcRing];              // the last MMAs that read a slot have completed
+  uint64_t done[2];                     // an accumulator's MMAs have completed
+  uint64_t empty[2];                    // an accumulator has been read by the four epilogue warps
   uint32_t tmem;
+  int zero_x0[kTcRing];                 // the column range a slot's zeros outside the image were written for
 };
 constexpr size_t kTcAOffset = (sizeof(TcSmem) + 127) / 128 * 128;
-constexpr size_t tc_smem_bytes(int dil) { return kTcAOffset + 3 * 4 * static_cast<size_t>(kTcTile + 2 * dil) * 16; }
+__host__ __device__ constexpr size_t tc_ring_bytes(int dil) { return kTcRing * 4 * static_cast<size_t>(kTcTile + 2 * dil) * 16; }
+constexpr size_t tc_smem_bytes(int dil) { return kTcAOffset + tc_ring_bytes(dil); }
 // ... and the folded last layer's weights after the ring (conv_tc_kernel<true>)
 constexpr size_t kTcLastBytes = 9 * 32 * sizeof(float);
 
@@ -796,6 +805,21 @@ __device__ __forceinline__ void tc_mma(uint32_t tmem, uint64_t ad, uint64_t bd, 
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
       "l"(ad), "l"(bd), "r"(kTcIdesc), "r"(accumulate)
+      : "memory");
+}
+
+// The same with the descriptors' low words (address and leading offset; the
+// high word is the same for every operand here), so that a step between the
+// operands of one row is one 32-bit addition.
+__device__ __forceinline__ uint32_t tc_desc_lo(uint32_t addr, uint32_t lbo) {
+  return ((addr & 0x3FFFFu) >> 4) | ((lbo >> 4) << 16);
+}
+__device__ __forceinline__ void tc_mma_lo(uint32_t tmem, uint32_t a, uint32_t b, uint32_t accumulate) {
+  constexpr uint32_t kHi = (128u >> 4) | (1u << 14);  // stride 128 bytes, version bits
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n mov.b64 da, {%1, %3};\n"
+      " mov.b64 db, {%2, %3};\n tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(tmem),
+      "r"(a), "r"(b), "r"(kHi), "r"(kTcIdesc), "r"(accumulate)
       : "memory");
 }
 
@@ -826,9 +850,39 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return l | (h << 16);
 }
 
-// One 32 -> 32 layer with ReLU: x, y NHWC BF16 (B, H, W, 32); wp the packed
-// weights [tap][chunk][out][8]; bias BF16.  Persistent over tiles; err gets
-// kErrTimeout if an MMA completion wait gives up.
+// A pixel's 32 channels: bias, ReLU, BF16, to the four planes of its row.
+__device__ __forceinline__ void tc_store_row(const float (&v)[32], const float* bias, uint4* dst, int W) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float o[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[e] = fmaxf(v[c * 8 + e] + bias[c * 8 + e], 0.0f);
+    dst[static_cast<int64_t>(c) * W] =
+        make_uint4(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]), pack_bf16x2(o[4], o[5]), pack_bf16x2(o[6], o[7]));
+  }
+}
+
+// One 32 -> 32 layer with ReLU: x, y BF16 in the layout of tc_act; wp the
+// packed weights [tap][chunk][out][8]; bias BF16.  Persistent over strips;
+// err gets kErrTimeout if a wait gives up.
+//
+// A work item is a strip: the output rows y0, y0 + dil, ..., of one image and
+// one 128-pixel column range (at most `strip` of them).  Output row y_k reads
+// input rows y_k - dil, y_k and y_k + dil, so consecutive rows of a strip
+// share two of their three input rows.  What bounds a row is the chain of its
+// steps (copy, MMAs, read-back, stores), so they run side by side: a copy
+// warp fills a ring of staged rows (four bulk copies each), one thread of
+// another warp issues a row's 18 MMAs into one of two accumulators, and the
+// four epilogue warps read the other back and store.  The staged rows of all
+// strips form one sequence (row s in slot s % kTcRing), so the copies run
+// ahead across strips.
+// (Copies by the block's threads, 16 bytes per instruction and 64 apart, and
+// one accumulator: 186, 186 and 201 us a layer on 64 images of 256^2 at
+// dilations 4, 16 and 64, 231 for the last; this form 109, 107, 143 and 158;
+// the layers' compulsory bytes take 80 and 63.  What is left is shared memory:
+// the MMAs read each staged row nine times, about 580 cycles a row.  Rings of
+// 4 and 6 rows: 719 and 751 us a batch against 676.)
+//
 // LAST: this is the network's last 32 -> 32 layer and the 32 -> 1 layer
 // after it is folded into its epilogue: since that layer has one output
 // channel, its output is y(p) = b + sum over taps of t_tap(p + offset_tap)
@@ -845,272 +899,389 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const __nv_bfloat16
                                                              __nv_bfloat16* __restrict__ y, int* err) {
   extern __shared__ __align__(1024) unsigned char tc_raw[];
   TcSmem& S = *reinterpret_cast<TcSmem*>(tc_raw);
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, lane = t & 31;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // uniform
   for (int i = t; i < kTcPacked / 8; i += kTcThreads)
     reinterpret_cast<uint4*>(S.b)[i] = __ldg(reinterpret_cast<const uint4*>(wp) + i);
   if (t < 32) S.bias[t] = __bfloat162float(bias[t]);
   // LAST: the 32 -> 1 layer's weights [tap][channel], after the ring
-  float* const w_last_s =
-      reinterpret_cast<float*>(tc_raw + kTcAOffset + 3 * 4 * static_cast<size_t>(kTcTile + 2 * dil) * 16);
+  float* const w_last_s = reinterpret_cast<float*>(tc_raw + kTcAOffset + tc_ring_bytes(dil));
   if (LAST)
     for (int i = t; i < 9 * 32; i += kTcThreads) w_last_s[i] = __bfloat162float(w_last[(i & 31) * 9 + (i >> 5)]);
   if (t == 0) {
-    mbar_init(&S.bar, 1);
+    for (int q = 0; q < kTcRing; ++q) {
+      mbar_init(&S.full[q], 1);
+      mbar_init(&S.free_[q], 1);
+      S.zero_x0[q] = -1;
+    }
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&S.done[q], 1);
+      mbar_init(&S.empty[q], 4);
+    }
     fence_mbar_init();
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_u32(&S.tmem))
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(smem_u32(&S.tmem))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the weights -> tensor core reads
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = S.tmem;
-  const int64_t n_pix = static_cast<int64_t>(B) * H * W;  // LAST: the T planes' stride
   const int nslot = kTcTile + 2 * dil;              // pixel slots of a staged row
   const uint32_t chunk_a = static_cast<uint32_t>(nslot) * 16;  // bytes between its 8-channel chunks
   uint4* const ring = reinterpret_cast<uint4*>(tc_raw + kTcAOffset);
-  const uint32_t a_base = smem_u32(ring), b_base = smem_u32(S.b);
   const int tiles_x = (W + kTcTile - 1) / kTcTile;
-  // Work items are strips: the output rows y0, y0 + dil, ..., of one image
-  // and one 128-pixel column range (at most `strip` of them).  Output row
-  // y_k reads input rows y_k - dil, y_k and y_k + dil, so consecutive rows of
-  // a strip share two of their three input rows: a ring of three staged rows
-  // holds them, and each tile after a strip's first stages one new row,
-  // while the tile before it is read back.
   const int per_class = (H + dil - 1) / dil;             // rows of the fullest residue class
   const int chunks = (per_class + strip - 1) / strip;
   const int n_strips = B * tiles_x * dil * chunks;
-  uint32_t phase = 0;
-  bool pending = false;  // an MMA group whose completion was not observed
-  // Stages input row ys of image img (zeros outside the image) for the
-  // column range starting at x0 into ring slot q, with asynchronous 16-byte
-  // copies: nothing passes through registers, so all of a row's copies are
-  // in flight at once.
-  auto stage = [&](int64_t img, int ys, int x0, int q) {
-    for (int sl = t; sl < nslot; sl += kTcThreads) {
-      const int xs = x0 - dil + sl;
-      const bool in = ys >= 0 && ys < H && xs >= 0 && xs < W;
-      const uint4* src = in ? reinterpret_cast<const uint4*>(x + (img + static_cast<int64_t>(ys) * W + xs) * 32)
-                            : reinterpret_cast<const uint4*>(x);
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        cp_async16(ring + (q * 4 + c) * nslot + sl, src + c, in ? 16u : 0u);
-    }
-  };
-  bool failed = false;
-  for (int item = blockIdx.x; item < n_strips && !failed; item += gridDim.x) {
+  // item -> its image's first row, first column, first output row, rows
+  auto item_of = [&](int item, int64_t& row0, int& x0, int& y0) {
     int rest = item;
     const int ch = rest % chunks;
     rest /= chunks;
     const int cls = rest % dil;
     rest /= dil;
-    const int xt = rest % tiles_x;
-    const int b = rest / tiles_x;
-    const int x0 = xt * kTcTile;
-    const int64_t img = static_cast<int64_t>(b) * H * W;  // first pixel of this sample
-    const int y0 = cls + ch * strip * dil;                 // first output row of the strip
-    if (y0 >= H) continue;
-    const int nrow = min(strip, (H - 1 - y0) / dil + 1);
-    // input row m of the strip (m = -1 .. nrow) is y0 + m * dil, in slot (m + 1) % 3
-    stage(img, y0 - dil, x0, 0);
-    stage(img, y0, x0, 1);
-    stage(img, y0 + dil, x0, 2);
-    for (int k = 0; k < nrow; ++k) {
-      const int yy = y0 + k * dil;
-      cp_async_wait_all();
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // staged rows -> tensor core reads
-      tc_fence_before();
-      __syncthreads();
-      if (t == 0) {
-        tc_fence_after();
-        uint32_t acc = 0;
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky) {
-          const int q = (k + ky) % 3;  // slot of input row k - 1 + ky
-#pragma unroll
-          for (int kx = 0; kx < 3; ++kx)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const uint32_t aa = a_base + ((q * 4 + 2 * h) * nslot + kx * dil) * 16;
-              const uint32_t bb = b_base + ((ky * 3 + kx) * 4 + 2 * h) * kTcChunkB;
-              tc_mma(tmem, tc_desc(aa, chunk_a, 128), tc_desc(bb, kTcChunkB, 128), acc);
-              acc = 1;
-            }
+    x0 = (rest % tiles_x) * kTcTile;
+    row0 = static_cast<int64_t>(rest / tiles_x) * H;
+    y0 = cls + ch * strip * dil;
+    return y0 < H ? min(strip, (H - 1 - y0) / dil + 1) : 0;
+  };
+  uint32_t g = 0;  // output rows so far: row g uses accumulator g % 2
+  if (warp == 5) {
+    // ---- copies: input rows y0 - dil, y0, ..., y0 + nrow dil of every strip
+    uint32_t st = 0;  // staged rows so far: row st in slot st % kTcRing
+    bool ok = true;
+    for (int item = blockIdx.x; item < n_strips && ok; item += gridDim.x) {
+      int64_t row0;
+      int x0, y0;
+      const int nrow = item_of(item, row0, x0, y0);
+      const int lo = max(0, dil - x0), hi = min(nslot, W - x0 + dil);  // slots inside the image
+      const uint32_t bytes = static_cast<uint32_t>(hi - lo) * 16;
+      for (int i = 0; nrow > 0 && i < nrow + 2; ++i, ++st) {
+        const uint32_t q = st % kTcRing;
+        if (st >= kTcRing) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&S.free_[q], (st / kTcRing - 1) & 1, err));
+          if (!ok) break;
         }
-        tc_commit(&S.bar);
-      }
-      pending = true;
-      const bool ok = __syncthreads_and(mbar_wait(&S.bar, phase, err));
-      if (!ok) {
-        failed = true;
-        break;
-      }
-      pending = false;
-      phase ^= 1u;
-      // the MMAs have read the ring: input row k + 2 goes into the slot of
-      // row k - 1 while this tile's accumulator is read back and stored
-      if (k + 1 < nrow) stage(img, yy + 2 * dil, x0, k % 3);
-      tc_fence_after();
-      float v[32];
-      tc_load32(tmem + (static_cast<uint32_t>(warp * 32) << 16), v);
-      const int px = x0 + warp * 32 + lane;
-      if (px < W && LAST) {
-        float h[32];
-#pragma unroll
-        for (int c = 0; c < 32; ++c) h[c] = __bfloat162float(__float2bfloat16_rn(fmaxf(v[c] + S.bias[c], 0.0f)));
-        float* T = reinterpret_cast<float*>(y) + img + static_cast<int64_t>(yy) * W + px;
-#pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-          float tt = 0.0f;
-#pragma unroll
-          for (int c = 0; c < 32; ++c) tt = fmaf(w_last_s[tap * 32 + c], h[c], tt);
-          T[tap * n_pix] = tt;
+        uint4* const dst = ring + q * 4 * nslot;
+        if (S.zero_x0[q] != x0) {  // columns outside the image are zero, whichever row the slot holds
+          for (int c = 0; c < 4; ++c) {
+            for (int sl = lane; sl < lo; sl += 32) dst[c * nslot + sl] = make_uint4(0u, 0u, 0u, 0u);
+            for (int sl = hi + lane; sl < nslot; sl += 32) dst[c * nslot + sl] = make_uint4(0u, 0u, 0u, 0u);
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the MMAs' reads
+          __syncwarp();
+          if (lane == 0) S.zero_x0[q] = x0;
+          __syncwarp();
         }
-      } else if (px < W) {
-        uint4* dst = reinterpret_cast<uint4*>(y + (img + static_cast<int64_t>(yy) * W + px) * 32);
+        if (lane == 0) {
+          const int yy = y0 + (i - 1) * dil;
+          if (yy >= 0 && yy < H) {
+            mbar_arrive_expect_tx(&S.full[q], 4 * bytes);
+            const uint4* src = reinterpret_cast<const uint4*>(x) + tc_act(row0 + yy, 0, W, x0 - dil + lo);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          float o[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) o[e] = fmaxf(v[c * 8 + e] + S.bias[c * 8 + e], 0.0f);
-          dst[c] = make_uint4(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]), pack_bf16x2(o[4], o[5]),
-                              pack_bf16x2(o[6], o[7]));
+            for (int c = 0; c < 4; ++c)
+              bulk_g2s(dst + c * nslot + lo, src + static_cast<int64_t>(c) * W, bytes, &S.full[q]);
+          } else {
+            mbar_arrive(&S.full[q]);  // a row outside the image is left out of the sums
+          }
         }
       }
     }
-    // the next strip's first rows overwrite every slot: all reads of this
-    // strip's last tile are done (its MMAs completed above), and the
-    // barrier at the next tile's start orders the copies after them
+    // no copy of this block is in flight at exit (they have all been waited
+    // for unless a wait gave up: bounded)
+    if (lane == 0)
+      for (uint32_t u = st > kTcRing ? st - kTcRing : 0; u < st; ++u)
+        mbar_wait(&S.full[u % kTcRing], (u / kTcRing) & 1, err);
+  } else if (warp == 4) {
+    // ---- MMAs, issued by one thread
+    if (lane == 0) {
+      const uint32_t a0 = tc_desc_lo(smem_u32(ring), chunk_a), b0 = tc_desc_lo(smem_u32(S.b), kTcChunkB);
+      const uint32_t step_h = 2 * nslot, step_slot = 4 * nslot;  // in 16-byte units
+      uint32_t st = 0;  // the strip's first staged row
+      bool ok = true;
+      for (int item = blockIdx.x; item < n_strips && ok; item += gridDim.x) {
+        int64_t row0;
+        int x0, y0;
+        const int nrow = item_of(item, row0, x0, y0);
+        if (nrow == 0) continue;
+        auto landed = [&](uint32_t u) { return mbar_wait(&S.full[u % kTcRing], (u / kTcRing) & 1, err); };
+        ok = landed(st) && landed(st + 1);
+        for (int k = 0; k < nrow && ok; ++k) {
+          if (!(ok = landed(st + k + 2))) break;
+          if (g >= 2 && !(ok = mbar_wait(&S.empty[g & 1], ((g >> 1) - 1) & 1, err))) break;
+          tc_fence_after();
+          const uint32_t d = tmem + 32 * (g & 1);
+          uint32_t acc = 0;
+#pragma unroll
+          for (int ky = 0; ky < 3; ++ky) {
+            const int yy = y0 + (k - 1 + ky) * dil;
+            if (yy < 0 || yy >= H) continue;
+            const uint32_t a_row = a0 + ((st + k + ky) % kTcRing) * step_slot;
+#pragma unroll
+            for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                tc_mma_lo(d, a_row + kx * dil + h * step_h, b0 + ((ky * 3 + kx) * 4 + 2 * h) * (kTcChunkB / 16), acc);
+                acc = 1;
+              }
+          }
+          tc_commit(&S.done[g & 1]);
+          tc_commit(&S.free_[(st + k) % kTcRing]);
+          if (k == nrow - 1) {
+            tc_commit(&S.free_[(st + k + 1) % kTcRing]);
+            tc_commit(&S.free_[(st + k + 2) % kTcRing]);
+          }
+          ++g;
+        }
+        st += nrow + 2;
+      }
+      // the last MMAs have completed before the tensor memory is released
+      if (g > 0) mbar_wait(&S.done[(g - 1) & 1], ((g - 1) >> 1) & 1, err);
+    }
+  } else {
+    // ---- epilogue: warp w reads TMEM lanes 32 w .. 32 w + 31 (lane = pixel) ----
+    const int64_t n_pix = static_cast<int64_t>(B) * H * W;  // LAST: the T planes' stride
+    bool ok = true;
+    for (int item = blockIdx.x; item < n_strips && ok; item += gridDim.x) {
+      int64_t row0;
+      int x0, y0;
+      const int nrow = item_of(item, row0, x0, y0);
+      const int px = x0 + warp * 32 + lane;
+      // reads row g's accumulator into v and gives it back
+      auto read = [&](float (&v)[32]) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&S.done[g & 1], (g >> 1) & 1, err))) return false;
+        tc_fence_after();
+        tc_load32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + 32 * (g & 1), v);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&S.empty[g & 1]);
+        ++g;
+        return true;
+      };
+      if (LAST) {
+        // two rows at a time: a read of the tap weights (72 of 16 bytes) serves
+        // two pixels, since the shared memory is what the MMAs' operands, the
+        // copies and these reads compete for
+        auto relu = [&](float (&v)[32]) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) v[c] = __bfloat162float(__float2bfloat16_rn(fmaxf(v[c] + S.bias[c], 0.0f)));
+        };
+        for (int k = 0; k < nrow && ok; k += 2) {
+          float h0[32], h1[32];
+          const bool two = k + 1 < nrow;
+          if (!(ok = read(h0))) break;
+          relu(h0);
+          if (two) {
+            if (!(ok = read(h1))) break;
+            relu(h1);
+          } else {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) h1[c] = 0.0f;
+          }
+          float* T = reinterpret_cast<float*>(y) + (row0 + y0 + k * dil) * W + px;
+          const int64_t down = static_cast<int64_t>(dil) * W;
+#pragma unroll
+          for (int tap = 0; tap < 9; ++tap) {
+            float t0 = 0.0f, t1 = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              const float4 w = reinterpret_cast<const float4*>(w_last_s)[tap * 8 + c];
+              t0 = fmaf(w.x, h0[4 * c], t0);
+              t1 = fmaf(w.x, h1[4 * c], t1);
+              t0 = fmaf(w.y, h0[4 * c + 1], t0);
+              t1 = fmaf(w.y, h1[4 * c + 1], t1);
+              t0 = fmaf(w.z, h0[4 * c + 2], t0);
+              t1 = fmaf(w.z, h1[4 * c + 2], t1);
+              t0 = fmaf(w.w, h0[4 * c + 3], t0);
+              t1 = fmaf(w.w, h1[4 * c + 3], t1);
+            }
+            if (px < W) {
+              T[tap * n_pix] = t0;
+              if (two) T[tap * n_pix + down] = t1;
+            }
+          }
+        }
+      } else {
+        for (int k = 0; k < nrow; ++k) {
+          float v[32];
+          if (!(ok = read(v))) break;
+          if (px < W) tc_store_row(v, S.bias, reinterpret_cast<uint4*>(y) + tc_act(row0 + y0 + k * dil, 0, W, px), W);
+        }
+      }
+    }
   }
-  cp_async_wait_all();  // no copy of this block is left in flight at exit
-  // an MMA whose completion was not seen is waited for once more (bounded)
-  // before its accumulator's tensor memory is released
-  if (pending) mbar_wait(&S.bar, phase, err);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem) : "memory");
   }
 }
 
 // The first layer (2 -> 32, ReLU) on the tensor cores: an implicit GEMM
 // with K = 2 channels x 9 taps = 18, padded with zeros to 32 (two MMAs of
-// K = 16).  A tile is 128 pixels of one image row (M = 128): each thread
-// gathers its pixel's 18 input values (BF16 NCHW; zeros outside the image)
-// into the A tile, K-major without swizzle like conv_tc_kernel's operands
-// (8-value chunks 128 x 16 bytes apart); the block packs the 32 x 18
-// weights the same way once ([chunk][out][8], zero-padded); the epilogue is
-// conv_tc_kernel's (bias, ReLU, BF16 NHWC).  (A CUDA-core form, one thread
-// per pixel, was bound by its 576 FP32 fused multiply-adds per pixel.)
+// K = 16).  A tile is 128 pixels of one image row (M = 128), one per thread:
+// the thread's 18 inputs, read in FP32 and rounded to BF16, go into the A
+// tile, K-major without swizzle like conv_tc_kernel's operands (8-value
+// chunks 128 x 16 bytes apart); the block packs the 32 x 18 weights the same
+// way once ([chunk][out][8], zero-padded); the epilogue is conv_tc_kernel's.
+// A block walks strips of rows y0, y0 + dil, ...: a thread reads 6 new inputs
+// per row and keeps the other 12, the A tile and the accumulator are double,
+// and a row's read-back and stores overlap the next row's MMAs.  (All 18
+// inputs of every pixel, one tile at a time, from a BF16 copy of the input
+// made by another pass: 119 + 10 us on 64 images of 256^2; this form 78.)
 constexpr int kTcFirstChunkA = kTcTile * 16;  // bytes between the A tile's 8-value chunks
 
 struct TcFirstSmem {
-  __nv_bfloat16 a[4 * kTcTile * 8];  // [chunk][pixel][8 values of k]
-  __nv_bfloat16 b[4 * 32 * 8];       // [chunk][out][8 values of k]
+  __nv_bfloat16 a[2][4 * kTcTile * 8];  // [chunk][pixel][8 values of k]
+  __nv_bfloat16 b[4 * 32 * 8];          // [chunk][out][8 values of k]
   float bias[32];
-  uint64_t bar;
+  uint64_t done[2];
   uint32_t tmem;
 };
 
-__global__ void __launch_bounds__(kTcThreads) conv_first_tc_kernel(const __nv_bfloat16* __restrict__ x,
-                                                                   const __nv_bfloat16* __restrict__ w,
-                                                                   const __nv_bfloat16* __restrict__ bias, int B,
-                                                                   int H, int W, int dil,
-                                                                   __nv_bfloat16* __restrict__ y, int* err) {
+__global__ void __launch_bounds__(kTcFirstThreads) conv_first_tc_kernel(const float* __restrict__ x,
+                                                                        const __nv_bfloat16* __restrict__ w,
+                                                                        const __nv_bfloat16* __restrict__ bias,
+                                                                        int B, int H, int W, int dil, int strip,
+                                                                        __nv_bfloat16* __restrict__ y, int* err) {
   __shared__ __align__(1024) TcFirstSmem S;
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // uniform
   // weights [chunk j][out n][e] = w[n][8 j + e] (k = channel * 9 + tap), zero past k = 17
-  for (int i = t; i < 4 * 32 * 8; i += kTcThreads) {
+  for (int i = t; i < 4 * 32 * 8; i += kTcFirstThreads) {
     const int e = i & 7, n = (i >> 3) & 31, j = i >> 8;
     const int k = 8 * j + e;
     S.b[i] = k < 18 ? w[n * 18 + k] : __float2bfloat16_rn(0.0f);
   }
   if (t < 32) S.bias[t] = __bfloat162float(bias[t]);
+#pragma unroll
+  for (int q = 0; q < 2; ++q)  // k = 24 .. 31 stay zero
+    reinterpret_cast<uint4*>(S.a[q])[3 * kTcTile + t] = make_uint4(0u, 0u, 0u, 0u);
   if (t == 0) {
-    mbar_init(&S.bar, 1);
+    mbar_init(&S.done[0], 1);
+    mbar_init(&S.done[1], 1);
     fence_mbar_init();
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_u32(&S.tmem))
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(smem_u32(&S.tmem))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = S.tmem;
-  const uint32_t a_base = smem_u32(S.a), b_base = smem_u32(S.b);
   const int tiles_x = (W + kTcTile - 1) / kTcTile;
-  const int n_tiles = B * H * tiles_x;
+  const int per_class = (H + dil - 1) / dil, chunks = (per_class + strip - 1) / strip;
+  const int n_strips = B * tiles_x * dil * chunks;
   const int64_t HW = static_cast<int64_t>(H) * W;
-  uint32_t phase = 0;
-  bool pending = false;  // an MMA group whose completion was not observed
-  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int row = tile / tiles_x;  // b * H + yy
-    const int x0 = (tile - row * tiles_x) * kTcTile;
-    const int yy = row % H;
-    const int b = row / H;
-    const int px = x0 + t;  // this thread's pixel
-    const __nv_bfloat16* xb = x + static_cast<int64_t>(b) * 2 * HW;
-    __align__(16) __nv_bfloat16 v[32];
+  uint32_t g = 0;  // rows so far: row g uses buffers g % 2
+  int64_t out_row = -1;  // the row whose accumulator has not been read back
+  int out_px = 0;
+  bool ok = true;
+  // reads row g - 1's accumulator back and stores its pixels
+  auto finish = [&]() {
+    if (out_row < 0) return true;
+    if (!__syncthreads_and(mbar_wait(&S.done[(g - 1) & 1], ((g - 1) >> 1) & 1, err))) return false;
+    tc_fence_after();
+    float acc[32];
+    tc_load32(tmem + (static_cast<uint32_t>(warp * 32) << 16) + 32 * ((g - 1) & 1), acc);
+    if (out_px < W) tc_store_row(acc, S.bias, reinterpret_cast<uint4*>(y) + tc_act(out_row, 0, W, out_px), W);
+    out_row = -1;
+    return true;
+  };
+  for (int item = blockIdx.x; item < n_strips && ok; item += gridDim.x) {
+    int rest = item;
+    const int ch = rest % chunks;
+    rest /= chunks;
+    const int cls = rest % dil;
+    rest /= dil;
+    const int px = (rest % tiles_x) * kTcTile + t;
+    const int b = rest / tiles_x;
+    const int y0 = cls + ch * strip * dil;
+    const int nrow = y0 < H ? min(strip, (H - 1 - y0) / dil + 1) : 0;
+    const float* xb = x + static_cast<int64_t>(b) * 2 * HW;
+    // inputs of three rows: in[channel][row][kx]
+    float in[2][3][3];
+    auto load = [&](int m, float (&dst)[2][3]) {  // row m of the strip
+      const int ii = y0 + m * dil;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = __float2bfloat16_rn(0.0f);
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx) {
+          const int jj = px + dil * (kx - 1);
+          dst[c][kx] = 0.0f;
+          if (px < W && ii >= 0 && ii < H && jj >= 0 && jj < W)
+            dst[c][kx] = __ldg(xb + c * HW + static_cast<int64_t>(ii) * W + jj);
+        }
+    };
+    float r0[2][3], r1[2][3], next[2][3];
+    load(-1, r0);
+    load(0, r1);
+    load(1, next);
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
-      for (int ky = 0; ky < 3; ++ky)
+      for (int kx = 0; kx < 3; ++kx) {
+        in[c][0][kx] = 0.0f;
+        in[c][1][kx] = r0[c][kx];
+        in[c][2][kx] = r1[c][kx];
+      }
+    for (int k = 0; k < nrow; ++k) {
+      const int q = g & 1;  // free: row g - 2 was read back before row g - 1 was issued
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
 #pragma unroll
         for (int kx = 0; kx < 3; ++kx) {
-          const int ii = yy + dil * (ky - 1), jj = px + dil * (kx - 1);
-          if (px < W && ii >= 0 && ii < H && jj >= 0 && jj < W)
-            v[c * 9 + ky * 3 + kx] = xb[c * HW + static_cast<int64_t>(ii) * W + jj];
+          in[c][0][kx] = in[c][1][kx];
+          in[c][1][kx] = in[c][2][kx];
+          in[c][2][kx] = next[c][kx];
         }
+      load(k + 2, next);
+      float v[24];
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      reinterpret_cast<uint4*>(S.a)[j * kTcTile + t] = *reinterpret_cast<const uint4*>(v + 8 * j);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor core reads
-    tc_fence_before();
-    __syncthreads();
-    if (t == 0) {
-      tc_fence_after();
+      for (int e = 0; e < 24; ++e) v[e] = e < 18 ? in[e / 9][(e % 9) / 3][e % 3] : 0.0f;
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        tc_mma(tmem, tc_desc(a_base + 2 * h * kTcFirstChunkA, kTcFirstChunkA, 128),
-               tc_desc(b_base + 2 * h * kTcChunkB, kTcChunkB, 128), h);
-      tc_commit(&S.bar);
-    }
-    pending = true;
-    const bool ok = __syncthreads_and(mbar_wait(&S.bar, phase, err));
-    if (!ok) break;
-    pending = false;
-    phase ^= 1u;
-    tc_fence_after();
-    float acc[32];
-    tc_load32(tmem + (static_cast<uint32_t>(warp * 32) << 16), acc);
-    const int po = x0 + warp * 32 + lane;  // TMEM lane = pixel
-    if (po < W) {
-      uint4* dst = reinterpret_cast<uint4*>(y + (static_cast<int64_t>(b) * HW + static_cast<int64_t>(yy) * W + po) * 32);
+      for (int j = 0; j < 3; ++j)
+        reinterpret_cast<uint4*>(S.a[q])[j * kTcTile + t] =
+            make_uint4(pack_bf16x2(v[8 * j], v[8 * j + 1]), pack_bf16x2(v[8 * j + 2], v[8 * j + 3]),
+                       pack_bf16x2(v[8 * j + 4], v[8 * j + 5]), pack_bf16x2(v[8 * j + 6], v[8 * j + 7]));
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor core reads
+      tc_fence_before();
+      __syncthreads();
+      if (t == 0) {
+        tc_fence_after();
+        const uint32_t a_base = smem_u32(S.a[q]), b_base = smem_u32(S.b);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        float o[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] = fmaxf(acc[c * 8 + e] + S.bias[c * 8 + e], 0.0f);
-        dst[c] = make_uint4(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]), pack_bf16x2(o[4], o[5]),
-                            pack_bf16x2(o[6], o[7]));
+        for (int h = 0; h < 2; ++h)
+          tc_mma(tmem + 32 * q, tc_desc(a_base + 2 * h * kTcFirstChunkA, kTcFirstChunkA, 128),
+                 tc_desc(b_base + 2 * h * kTcChunkB, kTcChunkB, 128), h);
+        tc_commit(&S.done[q]);
       }
+      if (!(ok = finish())) {
+        ++g;  // this row's MMAs are waited for below
+        break;
+      }
+      out_row = static_cast<int64_t>(b) * H + y0 + k * dil;
+      out_px = px;
+      ++g;
     }
   }
-  // an MMA whose completion was not seen is waited for once more (bounded)
-  // before its accumulator's tensor memory is released
-  if (pending) mbar_wait(&S.bar, phase, err);
+  if (ok) finish();
+  // the last MMAs have completed before their tensor memory is released
+  // (after a wait that gave up: bounded)
+  if (g > 0) mbar_wait(&S.done[(g - 1) & 1], ((g - 1) >> 1) & 1, err);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem) : "memory");
   }
 }
 
@@ -1130,25 +1301,37 @@ __global__ void pack_tc_kernel(const float* __restrict__ p, int64_t off0, int64_
 // nine taps of T[tap][p + offset_tap] (zero outside the image), the planes
 // the last 32 -> 32 layer's epilogue wrote (conv_tc_kernel<true>); taps in
 // (ky, kx) order.  y FP32 (B, 1, H, W).
+// A thread sums four pixels, so that 36 loads are in flight.
+constexpr int kLastPix = 4;
+
 __global__ void __launch_bounds__(256) conv_last_sum_kernel(const float* __restrict__ T,
                                                             const __nv_bfloat16* __restrict__ bias, int B, int H,
                                                             int W, int dil, float* __restrict__ y) {
   const int HW = H * W;
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= HW) return;
   const int b = blockIdx.y;
-  const int i = p / W, j = p - i * W;
   const int64_t n_pix = static_cast<int64_t>(B) * HW;
   const float* Tb = T + static_cast<int64_t>(b) * HW;
-  float acc = __bfloat162float(bias[0]);
+  const float b0 = __bfloat162float(bias[0]);
+  float t[kLastPix][9];
 #pragma unroll
-  for (int ky = 0; ky < 3; ++ky)
+  for (int u = 0; u < kLastPix; ++u) {
+    const int p = (blockIdx.x * kLastPix + u) * 256 + threadIdx.x;
+    const int i = p / W, j = p - i * W;
 #pragma unroll
-    for (int kx = 0; kx < 3; ++kx) {
-      const int ii = i + dil * (ky - 1), jj = j + dil * (kx - 1);
-      if (ii >= 0 && ii < H && jj >= 0 && jj < W) acc += __ldg(Tb + (ky * 3 + kx) * n_pix + ii * W + jj);
+    for (int tap = 0; tap < 9; ++tap) {
+      const int ii = i + dil * (tap / 3 - 1), jj = j + dil * (tap % 3 - 1);
+      t[u][tap] = 0.0f;
+      if (p < HW && ii >= 0 && ii < H && jj >= 0 && jj < W) t[u][tap] = __ldg(Tb + tap * n_pix + ii * W + jj);
     }
-  y[static_cast<int64_t>(b) * HW + p] = acc;
+  }
+#pragma unroll
+  for (int u = 0; u < kLastPix; ++u) {
+    const int p = (blockIdx.x * kLastPix + u) * 256 + threadIdx.x;
+    float acc = b0;
+#pragma unroll
+    for (int tap = 0; tap < 9; ++tap) acc += t[u][tap];
+    if (p < HW) y[static_cast<int64_t>(b) * HW + p] = acc;
+  }
 }
 
 int ew_grid(int64_t n) {
@@ -1172,7 +1355,7 @@ struct WsNet {
   bool bf_stale = true;
   float* act[kLayers + 1] = {};  // act[0] unused (the caller's input); act[l + 1] = layer l output
   float* dbuf[2] = {};           // data-gradient ping-pong
-  __nv_bfloat16* hbf[3] = {};    // inference: input copy (NCHW) + ping-pong activations (NHWC)
+  __nv_bfloat16* hbf[3] = {};    // inference: [1], [2] ping-pong activations (layout of tc_act)
   __nv_bfloat16* wtc = nullptr;  // the 32 -> 32 layers' weights in the tensor-core layout
   int* err = nullptr;            // device-side wait that gave up (kErrTimeout)
   int tc_smem_sm = 0, tc_reserved = 0;  // shared memory per SM and reserved per block
@@ -1338,37 +1521,38 @@ int infer_bf16(WsNet& N, int B, const float* x, float* y, cudaStream_t s) {
     GK_TRY_CUDA(cudaGetLastError());
     N.bf_stale = false;
   }
-  const int64_t nin = static_cast<int64_t>(B) * 2 * N.H * N.W;
-  to_bf16_kernel<<<ew_grid(nin), 256, 0, s>>>(x, N.hbf[0], nin);
-  GK_TRY_CUDA(cudaGetLastError());
-  const dim3 pg((N.H * N.W + 255) / 256, B);
+  const dim3 pg((N.H * N.W + 256 * kLastPix - 1) / (256 * kLastPix), B);
   const int64_t tiles = static_cast<int64_t>(B) * N.H * ((N.W + kTcTile - 1) / kTcTile);
-  conv_first_tc_kernel<<<static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(tiles, 8 * sm_count()))),
-                         kTcThreads, 0, s>>>(N.hbf[0], N.pbf + N.off_w[0], N.pbf + N.off_b[0], B, N.H, N.W,
-                                             N.dil[0], N.hbf[1], N.err);
+  // strips as long as the work still gives every resident CTA about four of
+  // them (a batch of one image runs single rows, each reading its three input
+  // rows; large batches reuse rows along strips of up to 16), then evened out
+  // over the rows of a residue class
+  auto strip_for = [&](int grid, int dil) {
+    const int target = static_cast<int>(
+        std::max<int64_t>(1, std::min<int64_t>(kTcStripMax, tiles / (4 * static_cast<int64_t>(grid)))));
+    const int per_class = (N.H + dil - 1) / dil;
+    const int n_chunks = (per_class + target - 1) / target;
+    return (per_class + n_chunks - 1) / n_chunks;
+  };
+  // 8 resident blocks per SM: 64 of the 512 tensor-memory columns each
+  const int grid1 = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(tiles, 8 * sm_count())));
+  conv_first_tc_kernel<<<grid1, kTcFirstThreads, 0, s>>>(x, N.pbf + N.off_w[0], N.pbf + N.off_b[0], B, N.H, N.W,
+                                                         N.dil[0], strip_for(grid1, N.dil[0]), N.hbf[1], N.err);
   GK_TRY_CUDA(cudaGetLastError());
   const __nv_bfloat16* in = N.hbf[1];
   for (int l = 1; l < kLayers - 1; ++l) {
     __nv_bfloat16* out = N.hbf[1 + (l & 1)];
     // resident blocks per SM: shared memory is the limit (registers, warps
-    // and the 512 tensor-memory columns allow 16 blocks of 32 columns), and
+    // and the 512 tensor-memory columns allow 8 blocks of 64 columns), and
     // it depends on the dilation through the staged rows' width
     const size_t smem = tc_smem_bytes(N.dil[l]) + (l == kLayers - 2 ? kTcLastBytes : 0);
-    int per_sm = std::max(1, std::min(16, static_cast<int>(static_cast<size_t>(N.tc_smem_sm) / (smem + N.tc_reserved))));
+    int per_sm = std::max(1, std::min(8, static_cast<int>(static_cast<size_t>(N.tc_smem_sm) / (smem + N.tc_reserved))));
     // small batches keep three blocks per SM (the count the widest rows
     // allow): more blocks would shorten every block's strips, and each strip
     // stages two rows more than it computes
     if (tiles < 16 * 3 * static_cast<int64_t>(sm_count())) per_sm = std::min(per_sm, 3);
     const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(tiles, int64_t(per_sm) * sm_count())));
-    // strips as long as the work still gives every resident CTA about four
-    // of them (a batch of one image runs single rows, each staging its
-    // three input rows; large batches reuse rows along strips of up to 16),
-    // then evened out over the rows of a residue class
-    const int target = static_cast<int>(
-        std::max<int64_t>(1, std::min<int64_t>(kTcStripMax, tiles / (4 * static_cast<int64_t>(grid)))));
-    const int per_class = (N.H + N.dil[l] - 1) / N.dil[l];
-    const int n_chunks = (per_class + target - 1) / target;
-    const int strip = (per_class + n_chunks - 1) / n_chunks;
+    const int strip = strip_for(grid, N.dil[l]);
     // the last 32 -> 32 layer also folds in the 32 -> 1 layer: it writes the
     // nine tap planes (36 bytes per pixel, within the 64 of the buffer)
     if (l == kLayers - 2)
@@ -1429,7 +1613,6 @@ extern "C" int gk_wsnet_create(int32_t H, int32_t W, int32_t batch_max, const in
   for (int l = 1; l <= kLayers; ++l)
     GK_TRY(dalloc_n(&N->act[l], l < kLayers ? big : static_cast<size_t>(batch_max) * img, by));
   for (float** q : {&N->dbuf[0], &N->dbuf[1]}) GK_TRY(dalloc_n(q, big, by));
-  GK_TRY(dalloc_n(&N->hbf[0], static_cast<size_t>(batch_max) * 2 * img, by));
   GK_TRY(dalloc_n(&N->hbf[1], big, by));
   GK_TRY(dalloc_n(&N->hbf[2], big, by));
   GK_TRY(dalloc_n(&N->wtc, static_cast<size_t>(kTcMidLayers) * kTcPacked, by));
