@@ -5,6 +5,9 @@
 // and read across the cluster (distributed shared memory), the other
 // vectors in registers of the thread that owns the row, and the cluster's
 // hardware barrier between the phases.
+// These kernels take the matrices whose halo (the other CTAs' rows a CTA's
+// rows refer to) does not fit its shared memory; the others run grid_cg.cu's
+// kernels on the same cluster, planned and launched from here.
 //
 // Small systems are latency-bound: the graph form spends a few microseconds
 // per kernel launch and per grid-wide reduction, three times per iteration,
@@ -690,10 +693,12 @@ int cluster_cg_plan(Solver* S) {
   S->cl_stage = stage;
   S->cl_nnz = stage ? static_cast<int>(most) : 0;
   S->cl_smem = smem;
-  return GK_OK;
+  // the halo form of the same cluster, where the halos fit shared memory
+  return grid_cg_plan(S, true);
 }
 
 int cluster_cg_solve(Solver* S, cudaStream_t s) {
+  if (S->gr_grid > 0) return grid_cg_solve(S, true, s);
   ClusterArgs a;
   a.rowptr = S->A->rowptr;
   a.col = S->A->col;

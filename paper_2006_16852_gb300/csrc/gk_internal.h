@@ -392,9 +392,11 @@ int cluster_cg_solve(Solver* S, cudaStream_t s);
 
 // CG (32,769 .. 262,144 rows) and BiCGSTAB (from 32,769 rows to 1,024 per SM)
 // of a mid-size system with rows of at most 64 entries, in one cooperative
-// launch with grid-wide reductions (grid_cg.cu).
-int grid_cg_plan(Solver* S);
-int grid_cg_solve(Solver* S, cudaStream_t s);
+// launch with grid-wide reductions (grid_cg.cu); cluster: the same kernels on
+// one 16-CTA cluster, for the small systems of cluster_cg.cu whose halos fit
+// shared memory (gr_grid > 0 after the plan).
+int grid_cg_plan(Solver* S, bool cluster);
+int grid_cg_solve(Solver* S, bool cluster, cudaStream_t s);
 
 // Restarted GMRES (gmres.cu).
 int gmres_generate(Solver* S);

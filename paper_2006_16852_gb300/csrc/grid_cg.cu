@@ -1,7 +1,8 @@
 // grid_cg.cu -- the whole preconditioned CG or BiCGSTAB solve (Section 3.1,
-// criteria of Section 2.5) of a mid-size system in ONE cooperative launch:
-// one CTA per SM, every CTA resident for the whole solve, the phases
-// separated by grid-wide reductions that are the grid's only barriers.
+// criteria of Section 2.5) in ONE launch whose CTAs are resident for the whole
+// solve, the phases separated by reductions over all CTAs that are the only
+// barriers: a cooperative launch of one CTA per SM for mid-size systems, a
+// 16-CTA thread-block cluster for small ones.
 //
 // Between the cluster form's sizes and a few hundred thousand rows, an
 // iteration of the graph form is bound by launch and reduction latency (~20
@@ -35,7 +36,7 @@
 // 17,900 cycles: direction 1,060, SpMV 2,400, update 1,440 (these three are
 // near the FP64 pipe's time for them), and per reduction 1,200 for the CTA's
 // sum, 2,300 - 3,700 until the last CTA's word is there, 990 for the sum of
-// the words, 980 for a division.  A dependent FP64 add takes 68 cycles, a
+// the words, 980 for a division (260 where none is left).  A dependent FP64 add takes 68 cycles, a
 // butterfly step 145, and a warp instruction holds its quarter of the SM's
 // FP64 pipe for about 64 cycles whatever its lanes do: hence one warp per
 // value in a reduction (a quarter each) and scalars derived by one thread
@@ -43,6 +44,15 @@
 // per iteration; before: an arrival counter and a release word per barrier,
 // vectors re-read from L2); BiCGSTAB, 201 x 199: 10.1 -> 4.2 ms (graph form
 // before).
+//
+// Small systems (the cluster sizes of cluster_cg.cu, whose kernels keep the
+// matrices whose halo does not fit): the same kernels on 16 CTAs, the
+// reductions' words pushed straight into every CTA's shared memory
+// (distributed shared memory) and polled there; the vectors' words stay in
+// L2, fetched while a reduction is in flight.  CG, Jacobi, Poisson 64 x 64 to
+// 1e-12: 1.40 -> 1.10 ms (6.0 -> 4.7 us per iteration; before: three cluster
+// barriers, p gathered across the cluster), 128 x 128 diffusion 4.64 -> 3.82
+// ms, BiCGSTAB 128 x 128 3.37 -> 2.68 ms.
 //
 // Every wait is bounded: one that gives up sets the error bit and an abort
 // word that ends every other CTA's waits at once, so the launch always
@@ -71,6 +81,7 @@ constexpr int kGrMaxK = 3;               // values per reduction
 // 21,400 cycles per iteration with 1 copy, 17,900 with 8, 18,400 with 19,
 // 18,500 with one per CTA, whose stores cost more than the polls save).
 constexpr int kGrCopies = 8;
+constexpr int kGrClusterCtas = 16;
 constexpr int kGrPlanThreads = 1024;
 
 struct GridArgs {
@@ -113,8 +124,35 @@ __device__ __forceinline__ double load_word(const ulonglong2* p, unsigned long l
 struct GridRed {
   double part[kGrMaxK][kGrThreads];
   double tot[kGrMaxK];
+  // CLUSTER: the CTAs' sums, pushed by their owners: each double as two 8-byte
+  // words {half, sequence number}, zero (no number) at the start
+  unsigned long long push[2][kGrMaxK][kGrClusterCtas][2];
   int ok;
 };
+
+// An 8-byte store into another CTA's shared memory (cluster address), and the
+// owner's load of it; each 8-byte word arrives whole.
+__device__ __forceinline__ void push_word(uint32_t addr, uint32_t half, uint32_t seq) {
+  asm volatile("{\n .reg .b64 w;\n mov.b64 w, {%1, %2};\n st.relaxed.cluster.shared::cluster.b64 [%0], w;\n}\n" ::"r"(addr),
+               "r"(half), "r"(seq)
+               : "memory");
+}
+__device__ __forceinline__ uint2 pushed_word(const unsigned long long* p) {
+  uint2 w;
+  asm volatile("{\n .reg .b64 w;\n ld.relaxed.cluster.shared::cta.b64 w, [%2];\n mov.b64 {%0, %1}, w;\n}\n"
+               : "=r"(w.x), "=r"(w.y)
+               : "r"(smem_u32(p))
+               : "memory");
+  return w;
+}
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 // Bounds a polling loop: true when the wait has to be given up (this one's
 // limit, or another wait's).
@@ -163,13 +201,13 @@ __device__ __forceinline__ void fetch_halo(const GridArgs& a, GridRed& red, cons
   }
 }
 
-// Sums v over the grid; then thread 0 of warp k < K of every CTA runs
-// post(k, totals) (the iteration's scalars are derived once per CTA, in
+// Sums v over the grid; then lanes 0 and 1 of warp k < K of every CTA run
+// post(k, lane, totals) (the iteration's scalars are derived once per CTA, in
 // parallel where they are independent: FP64 divisions and square roots are
-// long); false if the solve is being aborted.  Warp k sums value k: 8
+// long, and two quotients in two lanes take the time of one); false if the solve is being aborted.  Warp k sums value k: 8
 // threads' values per lane, one butterfly, then the CTAs' words, 5 per lane,
 // and one butterfly.  Meanwhile the other warps run idle(32 K).
-template <int K, typename Idle, typename Post>
+template <bool CLUSTER, int K, typename Idle, typename Post>
 __device__ __forceinline__ bool grid_total(const GridArgs& a, GridRed& red, unsigned long long& seq,
                                            const double (&v)[K], Idle idle, Post post) {
   // the warp's index from lane 0, so that the branch on it is uniform: the
@@ -193,48 +231,72 @@ __device__ __forceinline__ bool grid_total(const GridArgs& a, GridRed& red, unsi
     }
     double s[1] = {u[0]};
     warp_sum<1, double>(s);
-    if (lane < kGrCopies) store_word(a.words + lane * copy + slot + blockIdx.x, s[0], seq);
-    __syncwarp();
-    const ulonglong2* words = a.words + static_cast<int>(blockIdx.x % kGrCopies) * copy + slot;
     GrWait wait;
     bool ok = true;
-    double c[kGrMaxCtas / 32];
-    bool got[kGrMaxCtas / 32];
-#pragma unroll
-    for (int j = 0; j < kGrMaxCtas / 32; ++j) {
-      c[j] = 0.0;
-      got[j] = lane + 32 * j >= G;
-    }
-    for (;;) {
-      bool here = true;
-#pragma unroll
-      for (int j = 0; j < kGrMaxCtas / 32; ++j) {
-        if (!got[j]) {
-          unsigned long long q;
-          c[j] = load_word(words + lane + 32 * j, q);
-          got[j] = q == seq;
+    if constexpr (CLUSTER) {
+      const uint32_t seq32 = static_cast<uint32_t>(seq);
+      unsigned long long(*slot)[2] = red.push[seq & 1][warp];
+      if (lane < kGrClusterCtas) {
+        const uint32_t to = cluster_addr(slot[blockIdx.x], static_cast<uint32_t>(lane));
+        push_word(to, static_cast<uint32_t>(__double2loint(s[0])), seq32);
+        push_word(to + 8, static_cast<uint32_t>(__double2hiint(s[0])), seq32);
+      }
+      uint2 w0, w1;
+      for (;;) {
+        w0 = pushed_word(&slot[lane & (kGrClusterCtas - 1)][0]);
+        w1 = pushed_word(&slot[lane & (kGrClusterCtas - 1)][1]);
+        if (__all_sync(0xffffffffu, w0.y == seq32 && w1.y == seq32)) break;
+        const int stop = lane == 0 ? static_cast<int>(wait.give_up(a)) : 0;
+        if (__shfl_sync(0xffffffffu, stop, 0)) {
+          ok = false;
+          break;
         }
       }
+      s[0] = __hiloint2double(static_cast<int>(w1.x), static_cast<int>(w0.x));
 #pragma unroll
-      for (int j = 0; j < kGrMaxCtas / 32; ++j) here = here && got[j];
-      if (__all_sync(0xffffffffu, here)) break;
-      const int stop = lane == 0 ? static_cast<int>(wait.give_up(a)) : 0;
-      if (__shfl_sync(0xffffffffu, stop, 0)) {
-        ok = false;
-        break;
+      for (int o = kGrClusterCtas / 2; o > 0; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+    } else {
+      if (lane < kGrCopies) store_word(a.words + lane * copy + slot + blockIdx.x, s[0], seq);
+      __syncwarp();
+      const ulonglong2* words = a.words + static_cast<int>(blockIdx.x % kGrCopies) * copy + slot;
+      double c[kGrMaxCtas / 32];
+      bool got[kGrMaxCtas / 32];
+#pragma unroll
+      for (int j = 0; j < kGrMaxCtas / 32; ++j) {
+        c[j] = 0.0;
+        got[j] = lane + 32 * j >= G;
       }
-    }
-    s[0] = c[0];
+      for (;;) {
+        bool here = true;
 #pragma unroll
-    for (int j = 1; j < kGrMaxCtas / 32; ++j) s[0] += c[j];
-    warp_sum<1, double>(s);
+        for (int j = 0; j < kGrMaxCtas / 32; ++j) {
+          if (!got[j]) {
+            unsigned long long q;
+            c[j] = load_word(words + lane + 32 * j, q);
+            got[j] = q == seq;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kGrMaxCtas / 32; ++j) here = here && got[j];
+        if (__all_sync(0xffffffffu, here)) break;
+        const int stop = lane == 0 ? static_cast<int>(wait.give_up(a)) : 0;
+        if (__shfl_sync(0xffffffffu, stop, 0)) {
+          ok = false;
+          break;
+        }
+      }
+      s[0] = c[0];
+#pragma unroll
+      for (int j = 1; j < kGrMaxCtas / 32; ++j) s[0] += c[j];
+      warp_sum<1, double>(s);
+    }
     if (lane == 0) {
       red.tot[warp] = s[0];
       if (!ok) red.ok = 0;
     }
     if (K > 1) asm volatile("bar.sync 1, %0;" ::"n"(32 * K) : "memory");
     else __syncwarp();
-    if (lane == 0) post(warp, red.tot);
+    if (lane < 2) post(warp, lane, red.tot);
   } else {
     idle(32 * K);
   }
@@ -303,16 +365,20 @@ struct GridRows {
   }
 };
 
-// The iteration's scalars, derived by one thread of each CTA.
+// The iteration's scalars, derived by one thread of each CTA.  A division or
+// a square root there is about 650 cycles that every thread waits for, so
+// beta's divisor is inverted along with an earlier quotient, in another lane
+// (scale), and a norm's square root is taken only where the criteria may
+// hold: rr > tol2 implies ||r|| > tol.
 struct GrScalars {
-  double rho, rho_prev, alpha, omega, beta, rnorm, snorm, rnorm0, bnorm, ref, tol;
+  double rho, rho_prev, alpha, omega, beta, scale, rr, ss, rnorm0, bnorm, ref, tol, tol2;
   long long iter, spmvs;
   int stop, half, om_stop;
 };
 
 __device__ __forceinline__ void gr_init_scalars(GrScalars& sc) {
-  sc.rnorm0 = sc.bnorm = sc.rnorm = sc.snorm = sc.rho = sc.tol = 0.0;
-  sc.ref = sc.alpha = sc.omega = sc.rho_prev = 1.0;
+  sc.rnorm0 = sc.bnorm = sc.rr = sc.ss = sc.rho = sc.tol = sc.tol2 = 0.0;
+  sc.ref = sc.alpha = sc.omega = sc.rho_prev = sc.scale = 1.0;
   sc.beta = 0.0;
   sc.iter = 0;
   sc.spmvs = 1;
@@ -321,18 +387,39 @@ __device__ __forceinline__ void gr_init_scalars(GrScalars& sc) {
   sc.om_stop = GK_STOP_NONE;
 }
 
+// The solve's shared state; CLUSTER: every CTA of the cluster has started (and
+// its words are clear) before any is written to.
+template <bool CLUSTER>
+__device__ __forceinline__ void gr_start(GrScalars& sc, GridRed& red) {
+  if (threadIdx.x == 0) {
+    gr_init_scalars(sc);
+    red.ok = 1;
+  }
+  if constexpr (CLUSTER) {
+    unsigned long long* w = &red.push[0][0][0][0];
+    for (int i = threadIdx.x; i < 2 * kGrMaxK * kGrClusterCtas * 2; i += kGrThreads) w[i] = 0ull;
+    cluster_barrier();
+  } else {
+    __syncthreads();
+  }
+}
+
 // ||r0||^2 and ||b||^2 to the reference norm and the tolerance
 __device__ __forceinline__ void gr_setup_norms(GrScalars& sc, const double* tt, int rel_to_b, double factor) {
+  sc.rr = tt[0];
   sc.rnorm0 = sqrt(tt[0]);
   sc.bnorm = sqrt(tt[1]);
   double ref = rel_to_b ? sc.bnorm : sc.rnorm0;
   if (ref == 0.0) ref = 1.0;
   sc.ref = ref;
   sc.tol = factor * ref;
-  sc.rnorm = sc.rnorm0;
+  sc.tol2 = sc.tol * sc.tol * (1.0 + 0x1p-49);  // the margin covers the roundings of the product and the square root
 }
 
-__device__ __forceinline__ int gr_criteria(const GrScalars& sc, double rn, long long k, long long max_iters) {
+// The criteria on a squared norm: NaN, residual, iteration count.
+__device__ __forceinline__ int gr_criteria(const GrScalars& sc, double rr, long long k, long long max_iters) {
+  if (rr > sc.tol2 && isfinite(rr)) return k >= max_iters ? GK_STOP_MAX_ITERS : GK_STOP_NONE;
+  const double rn = sqrt(rr);
   if (!isfinite(rn)) return GK_STOP_NAN;
   if (rn <= sc.tol) return GK_STOP_CONVERGED;
   if (k >= max_iters) return GK_STOP_MAX_ITERS;
@@ -340,8 +427,8 @@ __device__ __forceinline__ int gr_criteria(const GrScalars& sc, double rn, long 
 }
 
 __device__ __forceinline__ void gr_store_state(SolverState* st, const GrScalars& sc, bool ok) {
-  st->rnorm = sc.rnorm;
-  st->snorm = sc.snorm;
+  st->rnorm = sqrt(sc.rr);
+  st->snorm = sqrt(sc.ss);
   st->rnorm0 = sc.rnorm0;
   st->bnorm = sc.bnorm;
   st->ref = sc.ref;
@@ -365,7 +452,7 @@ __device__ __forceinline__ void gr_store_state(SolverState* st, const GrScalars&
 //                                       the halo's z fetched meanwhile
 //   criteria; beta = rho' / rho
 // Shared memory: p of own rows and halo, z of the halo, the staged rows.
-template <int PK, int RPT, bool STAGE>
+template <int PK, int RPT, bool STAGE, bool CLUSTER>
 __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
   extern __shared__ double loc[];
   __shared__ GridRed red;
@@ -382,7 +469,6 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
   const long long max_iters = st->max_iters;
   const int rel_to_b = st->rel_to_b;
   unsigned long long seq = a.seq0;
-  auto nothing = [](int) {};
 
   double x[RPT], r[RPT], d[RPT], z[RPT], p[RPT];
   bool own[RPT];
@@ -397,11 +483,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
   }
   // x0 itself is not written before the end of the solve
   for (int h = t; h < H; h += kGrThreads) ph[h] = a.x[__ldg(A.halo + h)];
-  if (t == 0) {
-    gr_init_scalars(sc);
-    red.ok = 1;
-  }
-  __syncthreads();
+  gr_start<CLUSTER>(sc, red);
   unsigned long long zseq = a.seq0 + 1;  // sequence number of z_k's words
   bool ok;
   {
@@ -418,13 +500,13 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
       v[1] = fma(bi, bi, v[1]);
       v[2] = fma(r[u], z[u], v[2]);
     }
-    ok = grid_total<3>(
+    ok = grid_total<CLUSTER, 3>(
         a, red, seq, v, [&](int first) { fetch_halo(a, red, a.zw[0], zseq, A.halo, H, zh, first); },
-        [&](int w, const double* tt) {
-          if (w != 0) return;
+        [&](int w, int lane, const double* tt) {
+          if (w != 0 || lane != 0) return;
           gr_setup_norms(sc, tt, rel_to_b, factor);
           sc.rho = tt[2];
-          sc.stop = gr_criteria(sc, sc.rnorm, 0, max_iters);
+          sc.stop = gr_criteria(sc, sc.rr, 0, max_iters);
         });
   }
   for (long long k = 0; ok && sc.stop == GK_STOP_NONE; ++k) {
@@ -446,12 +528,18 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
       q[u] = A.apply(t + u * kGrThreads, loc);
       v[0] = fma(p[u], q[u], v[0]);
     }
-    if (!(ok = grid_total<1>(a, red, seq, v, nothing, [&](int, const double* tt) {
-            sc.spmvs += 1;
+    if (!(ok = grid_total<CLUSTER, 1>(a, red, seq, v, [](int) {}, [&](int, int lane, const double* tt) {
+            // lane 0: alpha = rho / sigma; lane 1: the next beta's factor 1 / rho
             const double sigma = tt[0];
+            const double q = (lane == 0 ? sc.rho : 1.0) / (lane == 0 ? sigma : sc.rho);
+            if (lane == 1) {
+              sc.scale = q;
+              return;
+            }
+            sc.spmvs += 1;
             if (!isfinite(sigma)) sc.stop = GK_STOP_NAN;
             else if (sigma <= 0.0) sc.stop = GK_STOP_BREAKDOWN;
-            else sc.alpha = sc.rho / sigma;
+            else sc.alpha = q;
           })))
       break;
     if (sc.stop != GK_STOP_NONE) break;
@@ -469,16 +557,17 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
       w[0] = fma(r[u], z[u], w[0]);
       w[1] = fma(r[u], r[u], w[1]);
     }
-    if (!(ok = grid_total<2>(
+    if (!(ok = grid_total<CLUSTER, 2>(
               a, red, seq, w, [&](int first) { fetch_halo(a, red, zw, zseq, A.halo, H, zh, first); },
-              [&](int warp, const double* tt) {
+              [&](int warp, int lane, const double* tt) {
+                if (lane != 0) return;
                 if (warp == 0) {
-                  sc.beta = tt[0] / sc.rho;
+                  sc.beta = tt[0] * sc.scale;
                   sc.rho = tt[0];
                 } else {
                   sc.iter += 1;
-                  sc.rnorm = sqrt(tt[1]);
-                  sc.stop = gr_criteria(sc, sc.rnorm, sc.iter, max_iters);
+                  sc.rr = tt[1];
+                  sc.stop = gr_criteria(sc, sc.rr, sc.iter, max_iters);
                 }
               })))
       break;
@@ -487,6 +576,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
   for (int u = 0; u < RPT; ++u)
     if (own[u]) a.x[row0 + t + u * kGrThreads] = x[u];
   if (blockIdx.x == 0 && t == 0) gr_store_state(st, sc, ok);
+  if (CLUSTER) cluster_barrier();  // no CTA leaves while others may still write to its shared memory
 }
 
 // BiCGSTAB (the Templates form, as the graph form computes it, with the
@@ -504,7 +594,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
 // reduction in every iteration and costs one SpMV in the last.)
 // Shared memory: the SpMV's input on own rows and halo; p^, z and v^ of the
 // halo; the staged rows.
-template <int PK, int RPT, bool STAGE>
+template <int PK, int RPT, bool STAGE, bool CLUSTER>
 __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
   extern __shared__ double loc[];
   __shared__ GridRed red;
@@ -536,17 +626,13 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
     if (own[u]) loc[l] = x[u];
   }
   for (int h = t; h < H; h += kGrThreads) in_h[h] = a.x[__ldg(A.halo + h)];
-  if (t == 0) {
-    gr_init_scalars(sc);
-    red.ok = 1;
-  }
-  __syncthreads();
+  gr_start<CLUSTER>(sc, red);
   // a fresh rho = r^.r either fails (NaN, zero) or yields the next beta
   auto new_rho = [&](double rho) {
     if (!isfinite(rho)) sc.stop = GK_STOP_NAN;
     else if (rho == 0.0) sc.stop = GK_STOP_BREAKDOWN;
     else {
-      sc.beta = (rho / sc.rho_prev) * (sc.alpha / sc.omega);
+      sc.beta = rho * sc.scale;  // scale = (alpha / omega) / the previous rho
       sc.rho = rho;
     }
   };
@@ -567,12 +653,12 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
       w[1] = fma(bi, bi, w[1]);
     }
     // r^ = r0: rho = r^.r is ||r0||^2
-    ok = grid_total<2>(
+    ok = grid_total<CLUSTER, 2>(
         a, red, seq, w, [&](int first) { fetch_halo(a, red, a.zw[0], wseq, A.halo, H, z_h, first); },
-        [&](int warp, const double* tt) {
-          if (warp != 0) return;
+        [&](int warp, int lane, const double* tt) {
+          if (warp != 0 || lane != 0) return;
           gr_setup_norms(sc, tt, rel_to_b, factor);
-          sc.stop = gr_criteria(sc, sc.rnorm, 0, max_iters);
+          sc.stop = gr_criteria(sc, sc.rr, 0, max_iters);
           if (sc.stop == GK_STOP_NONE) new_rho(tt[0]);
         });
   }
@@ -602,15 +688,21 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
         store_word(a.vw[cur] + row0 + l, vh[u], wseq);
         w[0] = fma(rh[u], v[u], w[0]);
       }
-      if (!(ok = grid_total<1>(
+      if (!(ok = grid_total<CLUSTER, 1>(
                 a, red, seq, w,
                 [&](int first) { fetch_halo(a, red, a.vw[cur], wseq, A.halo, H, vh_h, first); },
-                [&](int, const double* tt) {
-                  sc.spmvs += 1;
+                [&](int, int lane, const double* tt) {
+                  // lane 0: alpha = rho / r^.v; lane 1: 1 / r^.v for the next beta
                   const double rhv = tt[0];
+                  const double q = (lane == 0 ? sc.rho : 1.0) / rhv;
+                  if (lane == 1) {
+                    sc.scale = q;
+                    return;
+                  }
+                  sc.spmvs += 1;
                   if (!isfinite(rhv)) sc.stop = GK_STOP_NAN;
                   else if (rhv == 0.0) sc.stop = GK_STOP_BREAKDOWN;
-                  else sc.alpha = sc.rho / rhv;
+                  else sc.alpha = q;
                 })))
         break;
     }
@@ -638,17 +730,24 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
       }
       // warp 0: omega and its failures; warp 1: the half-step test, which
       // comes first where both hold
-      if (!(ok = grid_total<3>(a, red, seq, w, [](int) {}, [&](int warp, const double* tt) {
+      if (!(ok = grid_total<CLUSTER, 3>(a, red, seq, w, [](int) {}, [&](int warp, int lane, const double* tt) {
               if (warp == 0) {
+                // lane 0: omega = s.t / t.t; lane 1: the next beta's factor
+                // (alpha / omega) / rho = (1 / r^.v) (t.t / s.t)
+                const double q = tt[lane == 0 ? 0 : 2] / tt[lane == 0 ? 2 : 0];
+                if (lane == 1) {
+                  sc.scale *= q;
+                  return;
+                }
                 if (!isfinite(tt[2]) || !isfinite(tt[0])) sc.om_stop = GK_STOP_NAN;
                 else if (tt[2] == 0.0) sc.om_stop = GK_STOP_BREAKDOWN;
-                else sc.omega = tt[0] / tt[2];
-              } else if (warp == 1) {
-                sc.snorm = sqrt(tt[1]);
-                if (isfinite(sc.snorm) && sc.snorm <= sc.tol) {
+                else sc.omega = q;
+              } else if (warp == 1 && lane == 0) {
+                sc.ss = tt[1];
+                if (gr_criteria(sc, sc.ss, 0, 1) == GK_STOP_CONVERGED) {
                   sc.half = 1;
                   sc.iter += 1;
-                  sc.rnorm = sc.snorm;
+                  sc.rr = sc.ss;
                   sc.stop = GK_STOP_CONVERGED;
                 } else {
                   sc.spmvs += 1;
@@ -679,14 +778,15 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
         w[0] = fma(rh[u], r[u], w[0]);
         w[1] = fma(r[u], r[u], w[1]);
       }
-      if (!(ok = grid_total<2>(
-                a, red, seq, w, [&](int first) { fetch_halo(a, red, zw, wseq, A.halo, H, z_h, first); },
-                [&](int warp, const double* tt) {
-                  if (warp != 0) return;
+      if (!(ok = grid_total<CLUSTER, 2>(
+                a, red, seq, w,
+                [&](int first) { fetch_halo(a, red, zw, wseq, A.halo, H, z_h, first); },
+                [&](int warp, int lane, const double* tt) {
+                  if (warp != 0 || lane != 0) return;
                   sc.iter += 1;
                   sc.rho_prev = sc.rho;
-                  sc.rnorm = sqrt(tt[1]);
-                  int stop = gr_criteria(sc, sc.rnorm, sc.iter, max_iters);
+                  sc.rr = tt[1];
+                  int stop = gr_criteria(sc, sc.rr, sc.iter, max_iters);
                   if (stop == GK_STOP_NONE && sc.omega == 0.0) stop = GK_STOP_BREAKDOWN;
                   sc.stop = stop;
                   if (stop == GK_STOP_NONE) new_rho(tt[0]);
@@ -701,6 +801,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
     if (sc.stop == GK_STOP_NONE) sc.stop = sc.om_stop;
     gr_store_state(st, sc, ok);
   }
+  if (CLUSTER) cluster_barrier();
 }
 
 // The halo of every CTA: a bitmap of the columns of its rows that other CTAs
@@ -769,27 +870,47 @@ __global__ void __launch_bounds__(kGrPlanThreads) gr_halo_kernel(const int32_t* 
 
 using GrKernel = void (*)(GridArgs);
 
-template <int PK, bool STAGE>
+template <int PK, bool STAGE, bool CLUSTER>
 GrKernel pick_rpt(int kind, int rpt) {
   if (kind == GK_BICGSTAB) {
     switch (rpt) {
-      case 1: return bicg_grid_kernel<PK, 1, STAGE>;
-      case 2: return bicg_grid_kernel<PK, 2, STAGE>;
-      default: return bicg_grid_kernel<PK, 4, STAGE>;
+      case 1: return bicg_grid_kernel<PK, 1, STAGE, CLUSTER>;
+      case 2: return bicg_grid_kernel<PK, 2, STAGE, CLUSTER>;
+      default: return bicg_grid_kernel<PK, 4, STAGE, CLUSTER>;
     }
   }
   switch (rpt) {
-    case 1: return cg_grid_kernel<PK, 1, STAGE>;
-    case 2: return cg_grid_kernel<PK, 2, STAGE>;
-    case 4: return cg_grid_kernel<PK, 4, STAGE>;
-    default: return cg_grid_kernel<PK, 8, STAGE>;
+    case 1: return cg_grid_kernel<PK, 1, STAGE, CLUSTER>;
+    case 2: return cg_grid_kernel<PK, 2, STAGE, CLUSTER>;
+    case 4: return cg_grid_kernel<PK, 4, STAGE, CLUSTER>;
+    default: return cg_grid_kernel<PK, 8, STAGE, CLUSTER>;
   }
 }
 
-GrKernel pick(int kind, int pk, int rpt, bool stage) {
+template <bool CLUSTER>
+GrKernel pick_pk(int kind, int pk, int rpt, bool stage) {
   if (pk == PREC_SCALAR)
-    return stage ? pick_rpt<PREC_SCALAR, true>(kind, rpt) : pick_rpt<PREC_SCALAR, false>(kind, rpt);
-  return stage ? pick_rpt<PREC_NONE, true>(kind, rpt) : pick_rpt<PREC_NONE, false>(kind, rpt);
+    return stage ? pick_rpt<PREC_SCALAR, true, CLUSTER>(kind, rpt) : pick_rpt<PREC_SCALAR, false, CLUSTER>(kind, rpt);
+  return stage ? pick_rpt<PREC_NONE, true, CLUSTER>(kind, rpt) : pick_rpt<PREC_NONE, false, CLUSTER>(kind, rpt);
+}
+
+GrKernel pick(const Solver& S, int rpt, bool stage, bool cluster) {
+  return cluster ? pick_pk<true>(S.kind, S.pk, rpt, stage) : pick_pk<false>(S.kind, S.pk, rpt, stage);
+}
+
+cudaLaunchConfig_t cluster_config(size_t smem, cudaStream_t s, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kGrClusterCtas, 1, 1);
+  cfg.blockDim = dim3(kGrThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kGrClusterCtas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
 }
 
 // Dynamic shared memory a CTA may use (of 227 KB, next to the reductions' 6
@@ -798,18 +919,22 @@ constexpr size_t kGrSmemMax = 216 * 1024;
 
 }  // namespace
 
-int grid_cg_plan(Solver* S) {
+// cluster: the plan of the 16-CTA form (the caller has checked that the
+// cluster form applies); else of the cooperative grid.
+int grid_cg_plan(Solver* S, bool cluster) {
   S->gr_grid = 0;
   if ((S->kind != GK_CG && S->kind != GK_BICGSTAB) || S->pk == PREC_BLOCK) return GK_OK;
   const bool bi = S->kind == GK_BICGSTAB;
   const int64_t n = S->n;
-  if (n < kGrMinRows || n > kGrMaxRows) return GK_OK;
-  int coop = 0;
-  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, S->device) != cudaSuccess || !coop) {
-    cudaGetLastError();
-    return GK_OK;
+  if (!cluster) {
+    if (n < kGrMinRows || n > kGrMaxRows) return GK_OK;
+    int coop = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, S->device) != cudaSuccess || !coop) {
+      cudaGetLastError();
+      return GK_OK;
+    }
   }
-  const int G = sm_count();
+  const int G = cluster ? kGrClusterCtas : sm_count();
   const int64_t R = (n + G - 1) / G;
   int rpt = 1;
   while (static_cast<int64_t>(rpt) * kGrThreads < R) rpt *= 2;
@@ -819,7 +944,7 @@ int grid_cg_plan(Solver* S) {
   GK_TRY_CUDA(cudaMemcpy(rp.data(), S->A->rowptr, sizeof(int32_t) * rp.size(), cudaMemcpyDeviceToHost));
   int32_t longest = 0;
   for (int64_t i = 0; i < n; ++i) longest = std::max(longest, rp[i + 1] - rp[i]);
-  if (longest > kGrMaxRowLen) return GK_OK;
+  if (longest > kGrMaxRowLen && !cluster) return GK_OK;
   int64_t most = 0;
   for (int c = 0; c < G; ++c) {
     const int64_t lo = std::min<int64_t>(c * R, n), hi = std::min<int64_t>((c + 1) * R, n);
@@ -844,13 +969,19 @@ int grid_cg_plan(Solver* S) {
   const size_t staged = 12 * static_cast<size_t>(most) + 4 * static_cast<size_t>(R + 1);
   const bool stage = vectors + staged <= kGrSmemMax;
   const size_t smem = vectors + (stage ? staged : 0);
-  GrKernel k = pick(S->kind, S->pk, rpt, stage);
-  if (set_smem(k, smem) != GK_OK) {
-    cudaGetLastError();
-    return GK_OK;
+  GrKernel k = pick(*S, rpt, stage, cluster);
+  bool fits = set_smem(k, smem) == GK_OK;
+  if (fits && cluster) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = cluster_config(smem, nullptr, attr);
+    int clusters = 0;
+    fits = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+           cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) == cudaSuccess && clusters >= 1;
+  } else if (fits) {
+    int per_sm = 0;
+    fits = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kGrThreads, smem) == cudaSuccess && per_sm >= 1;
   }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kGrThreads, smem) != cudaSuccess || per_sm < 1) {
+  if (!fits) {
     cudaGetLastError();
     return GK_OK;
   }
@@ -874,7 +1005,7 @@ int grid_cg_plan(Solver* S) {
   return GK_OK;
 }
 
-int grid_cg_solve(Solver* S, cudaStream_t s) {
+int grid_cg_solve(Solver* S, bool cluster, cudaStream_t s) {
   const bool bi = S->kind == GK_BICGSTAB;
   GridArgs a;
   a.rowptr = S->A->rowptr;
@@ -908,10 +1039,16 @@ int grid_cg_solve(Solver* S, cudaStream_t s) {
   a.rows_per_cta = S->gr_rows;
   a.stage_nnz = S->gr_nnz;
   GK_TRY_CUDA(cudaMemsetAsync(a.abort_, 0, sizeof(unsigned int), s));
-  void* args[] = {&a};
-  GK_TRY_CUDA(cudaLaunchCooperativeKernel(
-      reinterpret_cast<const void*>(pick(S->kind, S->pk, S->gr_rpt, S->gr_stage)), dim3(S->gr_grid),
-      dim3(kGrThreads), args, S->gr_smem, s));
+  GrKernel k = pick(*S, S->gr_rpt, S->gr_stage, cluster);
+  if (cluster) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = cluster_config(S->gr_smem, s, attr);
+    GK_TRY_CUDA(cudaLaunchKernelEx(&cfg, k, a));
+  } else {
+    void* args[] = {&a};
+    GK_TRY_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k), dim3(S->gr_grid), dim3(kGrThreads), args,
+                                            S->gr_smem, s));
+  }
   return GK_OK;
 }
 

@@ -783,7 +783,7 @@ extern "C" int gk_solver_generate(gk_matrix hA, gk_precond hP, int32_t kind, con
     if (kind == GK_IR_CG && (rc = ir_generate(S))) break;
     if (kind == GK_GMRES && (rc = gmres_generate(S))) break;
     if ((kind == GK_CG || kind == GK_BICGSTAB) && (rc = cluster_cg_plan(S))) break;
-    if ((kind == GK_CG || kind == GK_BICGSTAB) && S->cl_lg < 0 && (rc = grid_cg_plan(S))) break;
+    if ((kind == GK_CG || kind == GK_BICGSTAB) && S->cl_lg < 0 && (rc = grid_cg_plan(S, false))) break;
   } while (false);
   if (prev != A->device) cudaSetDevice(prev);
   if (rc != GK_OK) return rc;
@@ -844,7 +844,7 @@ extern "C" int gk_solve(gk_solver h, const void* b, void* x, gk_status* status, 
         rc = cuda_error(e, "gk_solve: state init");
         break;
       }
-      if ((rc = grid_cg_solve(S, s))) break;
+      if ((rc = grid_cg_solve(S, false, s))) break;
       if ((rc = enqueue_final(*S, s))) break;
       form = GK_FORM_GRID;
     } else if (S->crit.check_every > 0) {
