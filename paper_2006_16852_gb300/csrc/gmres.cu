@@ -19,6 +19,7 @@
 #include <cmath>
 #include <cstring>
 #include <memory>
+#include <type_traits>
 
 #include "gk_device.cuh"
 #include "gk_internal.h"
@@ -30,6 +31,9 @@ namespace gk {
 constexpr int kGmresMaxDim = 128;
 constexpr int kGmresThreads = 256;
 constexpr int kDotThreads = 256;  // the dot-product sweep
+constexpr int kDotVecs = 8;       // vectors per sweep over the rows: one warp of the block sums each
+
+constexpr size_t kDotSmem = sizeof(double) * kDotVecs * kDotThreads;
 
 struct GmresState {
   double H[(kGmresMaxDim + 1) * kGmresMaxDim];  // H[i * m + j]
@@ -127,46 +131,83 @@ __global__ void __launch_bounds__(kGmresThreads) gm_precond_kernel(GmArgs a) {
   }
 }
 
-// h_i = V_i . w for every i <= j in one sweep: chunks of 8 vectors, each
-// chunk's FP64 partial sums per block (w is re-read per chunk, from L2); the
-// last block to arrive sums the block partials of every i in block order
-// (warp k takes i = k, k + 8, ...: lane l adds partials l, l + 32, ... into
-// four interleaved sums so that four loads are in flight, then the four
-// sums and one butterfly) and stores this pass's coefficients and H(i, j)
-// (the first pass sets it, the second adds).
+// h_i = V_i . w for every i <= j in one sweep: chunks of 8 vectors (w is
+// re-read per chunk, from L2), each chunk's per-thread sums reduced to one
+// partial per block; the last block to arrive sums the block partials of
+// every i in block order (warp k takes i = k, k + 16, ...: lane l adds
+// partials l, l + 32, ... into four interleaved sums so that four loads are
+// in flight, then the four sums and one butterfly) and stores this pass's
+// coefficients and H(i, j) (the first pass sets it, the second adds).
+// Bound by the FP64 pipe: (j + 1) n multiply-adds and, per block and vector, 7
+// adds and a butterfly in one warp.  The vectors of a sweep are a constant
+// number, so their loads carry no branch, and the branch around the
+// butterfly is uniform: under one on threadIdx.x a step of it took four
+// times as long.  At j = 20, n = 2^20: 70 -> 65 us, 41 of it
+// multiply-adds (one block of 512 threads per SM, whose reductions cost half,
+// left too few loads in flight: 110).
 __global__ void __launch_bounds__(kDotThreads) gm_dots_kernel(GmArgs a) {
-  __shared__ double scratch[8 * kDotThreads];
+  extern __shared__ double scratch[];  // [kDotVecs][kDotThreads]
   __shared__ unsigned int s_last;
   GmresState* s = a.gs;
   if (a.host && s->end) return;
   const int j = s->j;
   const int G = gridDim.x;
-  for (int c0 = 0; c0 <= j; c0 += 8) {
-    double acc[8];
+  const int lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x) >> 5, 0);  // uniform
+  // N vectors from c0 on; several rows per step for small N
+  auto sweep = [&](auto n_vec, int c0) {
+    constexpr int N = decltype(n_vec)::value;
+    constexpr int U = N >= 8 ? 1 : N >= 4 ? 2 : 4;  // rows per step
+    double acc[N];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = 0.0;
-    GM_FOR_ROWS(r) {
+    for (int k = 0; k < N; ++k) acc[k] = 0.0;
+    const double* Vc = a.V + static_cast<int64_t>(c0) * a.ldv;
+    const int stride = gridDim.x * kDotThreads;
+    int r = blockIdx.x * kDotThreads + threadIdx.x;
+    for (; r + (U - 1) * stride < a.n; r += U * stride) {
+      double wr[U], v[U][N];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        wr[u] = a.w[r + u * stride];
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[u][k] = Vc[k * a.ldv + r + u * stride];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < N; ++k) acc[k] = fma(v[u][k], wr[u], acc[k]);
+    }
+    for (; r < a.n; r += stride) {
       const double wr = a.w[r];
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (c0 + k <= j) acc[k] = fma(a.V[static_cast<int64_t>(c0 + k) * a.ldv + r], wr, acc[k]);
+      for (int k = 0; k < N; ++k) acc[k] = fma(Vc[k * a.ldv + r], wr, acc[k]);
     }
-    // block sums of the 8 values, warp k summing value k (lane l adds
-    // threads l, l + 32, ... in order, then one butterfly): block_sum's
-    // order, but eight warps share the slow FP64 adds instead of one
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 8; ++k) scratch[k * kDotThreads + threadIdx.x] = acc[k];
+    for (int k = 0; k < N; ++k) scratch[k * kDotThreads + threadIdx.x] = acc[k];
     __syncthreads();
-    const int wk = threadIdx.x >> 5, lk = threadIdx.x & 31;
-    if (wk < 8 && c0 + wk <= j) {
-      double v = scratch[wk * kDotThreads + lk];
-      for (int u = lk + 32; u < kDotThreads; u += 32) v += scratch[wk * kDotThreads + u];
+    if (warp < N) {
+      const double* p = scratch + warp * kDotThreads + lane;
+      double v[1] = {p[0]};
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lk == 0) a.dot_part[static_cast<int64_t>(c0 + wk) * G + blockIdx.x] = v;
+      for (int q = 1; q < kDotThreads / 32; ++q) v[0] += p[32 * q];
+      warp_sum<1, double>(v);
+      if (lane == 0) a.dot_part[static_cast<int64_t>(c0 + warp) * G + blockIdx.x] = v[0];
     }
+  };
+  int c = 0;
+  for (; c + 8 <= j + 1; c += 8) sweep(std::integral_constant<int, 8>(), c);
+  if (c + 4 <= j + 1) {
+    sweep(std::integral_constant<int, 4>(), c);
+    c += 4;
   }
+  switch (j + 1 - c) {
+    case 3: sweep(std::integral_constant<int, 3>(), c); break;
+    case 2: sweep(std::integral_constant<int, 2>(), c); break;
+    case 1: sweep(std::integral_constant<int, 1>(), c); break;
+    default: break;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     const unsigned int t = atomicAdd(a.dcounter, 1u);
@@ -175,7 +216,6 @@ __global__ void __launch_bounds__(kDotThreads) gm_dots_kernel(GmArgs a) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = warp; i <= j; i += kDotThreads / 32) {
     const double* p = a.dot_part + static_cast<int64_t>(i) * G;
     double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
@@ -187,76 +227,52 @@ __global__ void __launch_bounds__(kDotThreads) gm_dots_kernel(GmArgs a) {
       v3 += __ldcg(p + b + 96);
     }
     for (; b < G; b += 32) v0 += __ldcg(p + b);
-    double v = (v0 + v1) + (v2 + v3);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    double v[1] = {(v0 + v1) + (v2 + v3)};
+    warp_sum<1, double>(v);
     if (lane == 0) {
-      a.coef[i] = v;
-      if (s->pass == 0) s->H[i * a.m + j] = v;
-      else s->H[i * a.m + j] += v;
+      a.coef[i] = v[0];
+      if (s->pass == 0) s->H[i * a.m + j] = v[0];
+      else s->H[i * a.m + j] += v[0];
     }
   }
   if (threadIdx.x == 0) *a.dcounter = 0u;
 }
 
-// w -= sum_{i <= j} h_i V_i; on the second pass also ||w||^2 (the last block
-// stores ||w|| and advances the pass counter).
-__global__ void __launch_bounds__(kGmresThreads) gm_orth_kernel(GmArgs a) {
-  __shared__ double scratch[kRedScratch];
-  __shared__ double hs[kGmresMaxDim + 1];
-  GmresState* s = a.gs;
-  if (a.host && s->end) return;
-  const int j = s->j;
-  const bool last = s->pass == 1;
-  for (int i = threadIdx.x; i <= j; i += blockDim.x) hs[i] = a.coef[i];
-  __syncthreads();
-  double nn[1] = {0.0};
-  GM_FOR_ROWS(r) {
-    double wv = a.w[r];
-    for (int i = 0; i <= j; ++i) wv = fma(-hs[i], a.V[static_cast<int64_t>(i) * a.ldv + r], wv);
-    a.w[r] = wv;
-    nn[0] = fma(wv, wv, nn[0]);
-  }
-  double tot[1];
-  const bool lastblk = grid_sum<1, double>(nn, a.part, a.counter, scratch, tot);
-  if (lastblk && threadIdx.x == 0) {
-    if (last) s->hn = sqrt(tot[0]);
-    s->pass = last ? 0 : 1;
-  }
-}
+// h_{j+1,j} = ||w|| (hn); Givens rotations; residual estimate and criteria;
+// whether the cycle goes on (re-arms the WHILE node).  Run by the first warp
+// of the block that finished ||w||: column j of H and the previous rotations
+// are staged in shared memory by all lanes, lane 0 applies the rotations
+// there, all lanes write the column back.
+struct GmStepSmem {
+  double col[kGmresMaxDim + 1], cs[kGmresMaxDim], sn[kGmresMaxDim];
+};
 
-// h_{j+1,j} = ||w||; Givens rotations; residual estimate and criteria;
-// whether the cycle goes on (re-arms the WHILE node).  One warp: column j
-// of H and the previous rotations are staged in shared memory by all lanes,
-// lane 0 applies the rotations there, all lanes write the column back.
-__global__ void __launch_bounds__(32) gm_step_kernel(GmArgs a) {
-  __shared__ double col[kGmresMaxDim + 1], cs[kGmresMaxDim], sn[kGmresMaxDim];
+__device__ __forceinline__ void gm_step(const GmArgs& a, GmStepSmem& S) {
   GmresState* s = a.gs;
-  if (a.host && s->end) return;
   SolverState* st = a.st;
-  const int m = a.m, j = s->j, lane = threadIdx.x;
+  const int m = a.m, j = s->j, lane = threadIdx.x & 31;
   double* H = s->H;
-  for (int i = lane; i <= j; i += 32) col[i] = H[i * m + j];
+  for (int i = lane; i <= j; i += 32) S.col[i] = __ldcg(H + i * m + j);
   for (int i = lane; i < j; i += 32) {
-    cs[i] = s->cs[i];
-    sn[i] = s->sn[i];
+    S.cs[i] = s->cs[i];
+    S.sn[i] = s->sn[i];
   }
   __syncwarp();
   if (lane == 0) {
     const double hn = s->hn;
-    col[j + 1] = hn;
+    S.col[j + 1] = hn;
     for (int i = 0; i < j; ++i) {
-      const double x0 = col[i], x1 = col[i + 1];
-      col[i] = cs[i] * x0 + sn[i] * x1;
-      col[i + 1] = -sn[i] * x0 + cs[i] * x1;
+      const double x0 = S.col[i], x1 = S.col[i + 1];
+      S.col[i] = S.cs[i] * x0 + S.sn[i] * x1;
+      S.col[i + 1] = -S.sn[i] * x0 + S.cs[i] * x1;
     }
-    const double x0 = col[j], x1 = col[j + 1];
+    const double x0 = S.col[j], x1 = S.col[j + 1];
     const double d = hypot(x0, x1);
     const double c = d != 0.0 ? x0 / d : 1.0, sj = d != 0.0 ? x1 / d : 0.0;
     s->cs[j] = c;
     s->sn[j] = sj;
-    col[j] = d;
-    col[j + 1] = 0.0;
+    S.col[j] = d;
+    S.col[j + 1] = 0.0;
     const double gj = s->g[j];
     s->g[j + 1] = -sj * gj;
     s->g[j] = c * gj;
@@ -272,7 +288,40 @@ __global__ void __launch_bounds__(32) gm_step_kernel(GmArgs a) {
     if (!a.host) cudaGraphSetConditional(a.cond, s->end ? 0u : 1u);
   }
   __syncwarp();
-  for (int i = lane; i <= j + 1; i += 32) H[i * m + j] = col[i];
+  for (int i = lane; i <= j + 1; i += 32) H[i * m + j] = S.col[i];
+}
+
+// w -= sum_{i <= j} h_i V_i; on the second pass also ||w||^2: the last block
+// stores ||w|| and takes the step's decisions (gm_step; a launch of its own
+// for them took 11 us a step).
+__global__ void __launch_bounds__(kGmresThreads) gm_orth_kernel(GmArgs a) {
+  __shared__ double scratch[kRedScratch];
+  __shared__ double hs[kGmresMaxDim + 1];
+  __shared__ GmStepSmem step;
+  GmresState* s = a.gs;
+  if (a.host && s->end) return;
+  const int j = s->j;
+  const bool last = s->pass == 1;
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) hs[i] = a.coef[i];
+  __syncthreads();
+  double nn[1] = {0.0};
+  GM_FOR_ROWS(r) {
+    double wv = a.w[r];
+    for (int i = 0; i <= j; ++i) wv = fma(-hs[i], a.V[static_cast<int64_t>(i) * a.ldv + r], wv);
+    a.w[r] = wv;
+    nn[0] = fma(wv, wv, nn[0]);
+  }
+  double tot[1];
+  const bool lastblk = grid_sum<1, double>(nn, a.part, a.counter, scratch, tot);
+  if (!lastblk) return;
+  if (threadIdx.x == 0) {
+    if (last) s->hn = sqrt(tot[0]);
+    s->pass = last ? 0 : 1;
+  }
+  if (last && threadIdx.x < 32) {
+    __syncwarp();
+    gm_step(a, step);
+  }
 }
 
 // Unless the cycle ends: V_{j+1} = w / h_{j+1,j} and z = M^{-1} V_{j+1}
@@ -431,13 +480,11 @@ int gm_enqueue_step(const Solver& S, const GmresData& d, const GmArgs& a, cudaSt
   const int grid = gm_grid(S);
   GK_TRY(spmv_launch(*S.A, d.z, gm_epi(S, EPI_COPY, nullptr, d.w, FIN_NONE), s));
   for (int pass = 0; pass < 2; ++pass) {
-    gm_dots_kernel<<<d.dot_grid, kDotThreads, 0, s>>>(a);
+    gm_dots_kernel<<<d.dot_grid, kDotThreads, kDotSmem, s>>>(a);
     GK_TRY_CUDA(cudaGetLastError());
     gm_orth_kernel<<<d.grid, kGmresThreads, 0, s>>>(a);
     GK_TRY_CUDA(cudaGetLastError());
   }
-  gm_step_kernel<<<1, 32, 0, s>>>(a);
-  GK_TRY_CUDA(cudaGetLastError());
   GM_LAUNCH_PK(gm_next_kernel, grid, s, a);
   return GK_OK;
 }
