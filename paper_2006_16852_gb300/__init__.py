@@ -14,6 +14,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 from dataclasses import dataclass
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -203,6 +204,44 @@ def _check_vec(a, n: int, name: str, dtype_bits: int = 64):
         raise GkError(3, f"{name} must be float64, got {dt}")
 
 
+# The marshalling of a call whose vectors are contiguous float64 torch tensors,
+# without the general path's string comparisons and stream objects: a small
+# apply is bound by the host (5,000-row operators: 7.8 us a call, 4 of it
+# here, against about 2 for the launch).
+_tensor = _float64 = _raw_stream = None
+
+
+def _find_torch():
+    """Whether torch is loaded (the library never imports it on its own)."""
+    global _tensor, _float64, _raw_stream
+    torch = sys.modules.get("torch")
+    if torch is None or not hasattr(torch, "Tensor"):
+        return False
+    _tensor, _float64 = torch.Tensor, torch.float64
+    _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+        lambda i: torch.cuda.current_stream(i).cuda_stream)
+    return True
+
+
+def _fast_args(u, nu, v, nv, stream):
+    """(pointer of u, pointer of v, stream) of a call on two vectors, or None
+    where they are anything but contiguous float64 tensors of nu and nv
+    entries (the general path then checks them and names what is wrong)."""
+    if _tensor is None and not _find_torch():
+        return None
+    if not (type(u) is _tensor and type(v) is _tensor and u.dtype is _float64 and v.dtype is _float64
+            and u.numel() == nu and v.numel() == nv and u.is_contiguous() and v.is_contiguous()):
+        return None
+    if stream is None:
+        d = u.get_device()
+        if d < 0:
+            d = v.get_device()
+        st = _raw_stream(d) if d >= 0 else 0
+    else:
+        st = int(getattr(stream, "cuda_stream", stream))
+    return u.data_ptr(), v.data_ptr(), st
+
+
 class Matrix:
     """A CSR operator (library-owned copy) in one of the storage formats."""
 
@@ -234,6 +273,10 @@ class Matrix:
 
 def apply(A: Matrix, b, x, stream=None):
     """x = A b (Section 4.2)."""
+    f = _fast_args(b, A.n_cols, x, A.n_rows, stream)
+    if f is not None:
+        _check(lib().gk_apply(A.handle, *f))
+        return x
     _check_vec(b, A.n_cols, "b")
     _check_vec(x, A.n_rows, "x")
     _check(lib().gk_apply(A.handle, _ptr(b), _ptr(x), _stream(stream, b, x)))
@@ -251,6 +294,10 @@ def apply_dot(A: Matrix, b, x, u, result, stream=None):
 
 def apply_adv(alpha: float, A: Matrix, b, beta: float, x, stream=None):
     """x = alpha A b + beta x (Section 4.2)."""
+    f = _fast_args(b, A.n_cols, x, A.n_rows, stream)
+    if f is not None:
+        _check(lib().gk_apply_adv(float(alpha), A.handle, f[0], float(beta), f[1], f[2]))
+        return x
     _check_vec(b, A.n_cols, "b")
     _check_vec(x, A.n_rows, "x")
     _check(lib().gk_apply_adv(float(alpha), A.handle, _ptr(b), float(beta), _ptr(x), _stream(stream, b, x)))
@@ -288,6 +335,10 @@ def precond_generate(A: Matrix, block_size: int = 1, stream=None) -> Precond:
 
 def precond_apply(P: Precond, r, z, stream=None):
     """z = M^{-1} r."""
+    f = _fast_args(r, P.n, z, P.n, stream)
+    if f is not None:
+        _check(lib().gk_precond_apply(P.handle, *f))
+        return z
     _check_vec(r, P.n, "r")
     _check_vec(z, P.n, "z")
     _check(lib().gk_precond_apply(P.handle, _ptr(r), _ptr(z), _stream(stream, r, z)))

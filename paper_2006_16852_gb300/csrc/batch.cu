@@ -44,6 +44,15 @@ struct BatchClass {
   int k0 = 0;     // first position in the size order
   int count = 0;  // systems in the class
   int nmax = 0;   // rows of its largest system
+  int wmax = 0;   // its largest ELL width
+};
+
+// The vectors of the solve at hand, in device memory: the graph of a
+// configuration reads them from here, so that other vectors need no other
+// graph (building one takes about a millisecond).
+struct BatchIo {
+  const double* b;
+  double* x;
 };
 
 struct BatchArgs {
@@ -54,7 +63,8 @@ struct BatchArgs {
   const uint16_t* ell_col;  // local column indices
   const void* ell_val;      // values in the solve precision
   const float* ell_val32;   // FP32 copy of FP64 values (refinement inner solves)
-  const double* b;
+  const BatchIo* io;
+  const double* b;  // io's, read by each block
   double* x;
   gk_batch_status* st;
   unsigned int* next;  // this class's counter
@@ -557,6 +567,207 @@ __device__ void ir_system(const BatchArgs& a, unsigned char* smem, double* redd,
   }
 }
 
+// Sum of K FP32 values over the block, in every thread: a butterfly per warp,
+// then the warps' sums in order.  ws alternates between two buffers, so one
+// barrier is enough.
+template <bool WARP, int K>
+__device__ __forceinline__ void sum32(float (&v)[K], float (*ws)[2][8], int& parity) {
+  warp_sum<K, float>(v);
+  if (WARP) return;
+  float(*w)[8] = ws[parity];
+  parity ^= 1;
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) w[k][threadIdx.x >> 5] = v[k];
+  }
+  __syncthreads();
+  const int nw = blockDim.x >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    v[k] = w[k][0];
+    for (int q = 1; q < nw; ++q) v[k] += w[k][q];
+  }
+}
+
+// ir_system for systems of at most RPT * blockDim rows and W entries per row:
+// the same steps, with a thread's rows -- FP32 values, columns, and the
+// inner CG's r, q, d, p and inverse diagonal -- in its registers.  Only x
+// (FP64) and p are shared, so an inner iteration reads nothing but p from
+// shared memory and has three barriers; ir_system reads the matrix from
+// L1/L2 and five vectors from shared memory in every iteration, with eight
+// barriers, and its latency is what 10,000 systems of 36 to 1,024 rows wait
+// for: 5.76 -> 3.58 ms to 1e-12 with
+// one graph for all vectors (above).
+template <int RPT, int W, bool JAC, bool WARP>
+__device__ void ir_system_reg(const BatchArgs& a, unsigned char* smem, double* redd, double* sc, float (*ws)[2][8],
+                              int sys, int r0, int n) {
+  const SysMat<double> m64 = sys_mat<double>(a, sys, n);
+  const float* val32 = a.ell_val32 + a.ell_off[sys];
+  double* X = reinterpret_cast<double*>(smem);
+  float* P = reinterpret_cast<float*>(X + a.nmax);
+  const int t = threadIdx.x, T = blockDim.x, w = m64.w;
+  float val[RPT][W], dinv[RPT];
+  uint32_t col[RPT][(W + 1) / 2];  // two 16-bit columns each
+  bool own[RPT];
+#pragma unroll
+  for (int u = 0; u < RPT; ++u) {
+    const int i = t + u * T;
+    own[u] = i < n;
+    dinv[u] = 1.0f;
+    bool found = false;
+#pragma unroll
+    for (int k = 0; k < (W + 1) / 2; ++k) col[u][k] = 0u;
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      val[u][k] = 0.0f;
+      if (own[u] && k < w) {
+        const uint32_t c = m64.col[k * n + i];
+        val[u][k] = val32[k * n + i];
+        col[u][k / 2] |= c << (16 * (k & 1));
+        if (JAC && !found && c == static_cast<uint32_t>(i)) {  // padding repeats the row's own column after its entries
+          const double d = m64.val[k * n + i];
+          dinv[u] = d != 0.0 ? static_cast<float>(1.0 / d) : 1.0f;
+          found = true;
+        }
+      }
+    }
+    if (own[u]) X[i] = a.x[r0 + i];
+  }
+  auto column = [&](int u, int k) { return static_cast<int>((col[u][k / 2] >> (16 * (k & 1))) & 0xffffu); };
+  __syncthreads();
+  long long k_total = 0;
+  int steps = 0, stop = GK_STOP_NONE, parity = 0;
+  double rnorm = 0.0, ref = 1.0, tol = 0.0;
+  const int rel_to_b = a.rel_to_b;
+  for (;;) {
+    // FP64 residual and its norm (and ||b|| on the first step)
+    double r64[RPT], s2[2] = {0.0, 0.0};
+#pragma unroll
+    for (int u = 0; u < RPT; ++u) {
+      r64[u] = 0.0;
+      if (!own[u]) continue;
+      const int i = t + u * T;
+      double q = 0.0;
+#pragma unroll
+      for (int k = 0; k < W; ++k)
+        if (k < w) q = fma(__ldg(m64.val + k * n + i), X[column(u, k)], q);
+      const double bi = a.b[r0 + i];
+      r64[u] = bi - q;
+      s2[0] = fma(r64[u], r64[u], s2[0]);
+      s2[1] = fma(bi, bi, s2[1]);
+    }
+    double o[3];
+    const bool first = steps == 0;
+    const double ref_prev = ref;
+    reduce<WARP>(s2, redd, sc, o, [&](double(&v)[2], double(&out)[3]) {
+      const double rn = sqrt(v[0]);
+      double rf = ref_prev;
+      if (first) {
+        rf = rel_to_b ? sqrt(v[1]) : rn;
+        if (rf == 0.0) rf = 1.0;
+      }
+      out[0] = rn;
+      out[1] = rf;
+      out[2] = 1.0 / rn;
+    });
+    rnorm = o[0];
+    ref = o[1];
+    const double inv = o[2];
+    if (first) tol = a.factor * ref;
+    stop = sys_check(rnorm, tol, k_total, a.max_iters);
+    if (stop != GK_STOP_NONE || steps >= kBatchMaxOuter) {
+      if (stop == GK_STOP_NONE) stop = GK_STOP_MAX_ITERS;
+      break;
+    }
+    // FP32 inner CG on A d = r / ||r|| from d = 0
+    float r[RPT], d[RPT], p[RPT], q[RPT], v2[2] = {0.0f, 0.0f};
+#pragma unroll
+    for (int u = 0; u < RPT; ++u) {
+      r[u] = static_cast<float>(r64[u] * inv);
+      d[u] = 0.0f;
+      p[u] = JAC ? dinv[u] * r[u] : r[u];
+      if (own[u]) {
+        P[t + u * T] = p[u];
+        v2[0] = fmaf(r[u], p[u], v2[0]);
+        v2[1] = fmaf(r[u], r[u], v2[1]);
+      }
+    }
+    sum32<WARP, 2>(v2, ws, parity);
+    if (WARP) __syncwarp();  // P (the block's sum has a barrier)
+    float rho = v2[0];
+    const double red = fmax(a.inner_red, 0.5 * tol / rnorm);
+    // t <= tol2 for a float t exactly if t <= tol2 rounded down to a float
+    const float tol2 = __double2float_rd(red * red * static_cast<double>(v2[1]));
+    long long it = 0;
+    bool broke = false;
+    while (it < a.inner_max) {
+      float sg[1] = {0.0f};
+#pragma unroll
+      for (int u = 0; u < RPT; ++u) {
+        float s = 0.0f;
+#pragma unroll
+        for (int k = 0; k < W; ++k) s = fmaf(val[u][k], P[column(u, k)], s);
+        q[u] = s;
+        if (own[u]) sg[0] = fmaf(p[u], s, sg[0]);
+      }
+      sum32<WARP, 1>(sg, ws, parity);
+      if (!isfinite(sg[0]) || sg[0] <= 0.0f) {
+        broke = true;
+        break;
+      }
+      const float alpha = __fdiv_rn(rho, sg[0]);
+      float v[2] = {0.0f, 0.0f}, z[RPT];
+#pragma unroll
+      for (int u = 0; u < RPT; ++u) {
+        d[u] = fmaf(alpha, p[u], d[u]);
+        r[u] = fmaf(-alpha, q[u], r[u]);
+        z[u] = JAC ? dinv[u] * r[u] : r[u];
+        if (own[u]) {
+          v[0] = fmaf(r[u], z[u], v[0]);
+          v[1] = fmaf(r[u], r[u], v[1]);
+        }
+      }
+      sum32<WARP, 2>(v, ws, parity);
+      ++it;
+      if (!isfinite(v[0]) || !isfinite(v[1])) {
+        broke = true;
+        break;
+      }
+      if (v[1] <= tol2) break;
+      const float beta = __fdiv_rn(v[0], rho);
+      rho = v[0];
+      if (WARP) __syncwarp();
+#pragma unroll
+      for (int u = 0; u < RPT; ++u) {
+        p[u] = fmaf(beta, p[u], z[u]);
+        if (own[u]) P[t + u * T] = p[u];
+      }
+      if (WARP) __syncwarp();
+      else __syncthreads();
+    }
+    // x = x + ||r|| d in FP64
+#pragma unroll
+    for (int u = 0; u < RPT; ++u)
+      if (own[u]) X[t + u * T] = fma(rnorm, static_cast<double>(d[u]), X[t + u * T]);
+    __syncthreads();
+    k_total += it;
+    ++steps;
+    if (it == 0 || (broke && it <= 1)) {
+      stop = GK_STOP_BREAKDOWN;
+      break;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < RPT; ++u)
+    if (own[u]) a.x[r0 + t + u * T] = X[t + u * T];
+  if (t == 0 && a.st) {
+    a.st[sys].iters = static_cast<int32_t>(k_total);
+    a.st[sys].stop_reason = stop;
+    a.st[sys].rel_res = rnorm / ref;
+    a.st[sys].outer_iters = steps;
+  }
+}
+
 // Shared-memory bytes per row a block keeps for one system.
 __host__ __device__ constexpr int batch_row_bytes(int kind, bool jac, int el) {
   return kind == GK_CG ? el * (jac ? 5 : 4)
@@ -574,6 +785,8 @@ __global__ void __launch_bounds__(256) batch_kernel(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char bsm[];
   __shared__ double s_sc[4];
   __shared__ int s_k;
+  a.b = a.io->b;
+  a.x = a.io->x;
   T* V = reinterpret_cast<T*>(bsm);
   unsigned char* redp = bsm + batch_red_offset(KIND, JAC, static_cast<int>(sizeof(T)), a.nmax);
   T* red = reinterpret_cast<T*>(redp);
@@ -588,6 +801,29 @@ __global__ void __launch_bounds__(256) batch_kernel(BatchArgs a) {
     if constexpr (KIND == GK_CG) cg_system<T, JAC, WARP>(a, V, red, s_sc, sys, r0, n);
     else if constexpr (KIND == GK_BICGSTAB) bicg_system<T, JAC, WARP>(a, V, red, s_sc, sys, r0, n);
     else ir_system<JAC, WARP>(a, bsm, reinterpret_cast<double*>(redp), s_sc, sys, r0, n);
+  }
+}
+
+constexpr int kIrRegRowBytes = 12;  // x in FP64, p in FP32
+
+template <int RPT, int W, bool JAC, bool WARP>
+__global__ void __launch_bounds__(256) batch_ir_reg_kernel(BatchArgs a) {
+  extern __shared__ __align__(16) unsigned char bsm[];
+  __shared__ double s_sc[4];
+  __shared__ float s_ws[2][2][8];
+  __shared__ int s_k;
+  a.b = a.io->b;
+  a.x = a.io->x;
+  double* redd = reinterpret_cast<double*>(bsm + (static_cast<size_t>(kIrRegRowBytes) * a.nmax + 15) / 16 * 16);
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) s_k = static_cast<int>(atomicAdd(a.next, 1u));
+    __syncthreads();
+    const int k = s_k;
+    if (k >= a.count) break;
+    const int sys = a.order[a.k0 + k];
+    const int r0 = a.sys_ptr[sys], n = a.sys_ptr[sys + 1] - r0;
+    ir_system_reg<RPT, W, JAC, WARP>(a, bsm, redd, s_sc, s_ws, sys, r0, n);
   }
 }
 
@@ -649,6 +885,31 @@ BatchFn pick_kernel(int dtype, int kind, bool jac, int threads) {
   return dtype == GK_F32 ? pick_t<float>(kind, jac, warp) : pick_t<double>(kind, jac, warp);
 }
 
+// The register form of the refinement: rows per thread up to 8 (5 entries a
+// row) or 4 (8 entries), which the registers hold; null where a class's
+// systems are longer or wider for their block.
+template <int RPT, int W>
+BatchFn pick_ir_reg(bool jac, bool warp) {
+  if (jac) return warp ? batch_ir_reg_kernel<RPT, W, true, true> : batch_ir_reg_kernel<RPT, W, true, false>;
+  return warp ? batch_ir_reg_kernel<RPT, W, false, true> : batch_ir_reg_kernel<RPT, W, false, false>;
+}
+
+BatchFn pick_ir_reg(int nmax, int wmax, bool jac, int threads) {
+  const bool warp = threads == 32;
+  const int rpt = (nmax + threads - 1) / threads;
+  if (wmax <= 5) {
+    if (rpt <= 1) return pick_ir_reg<1, 5>(jac, warp);
+    if (rpt <= 2) return pick_ir_reg<2, 5>(jac, warp);
+    if (rpt <= 4) return pick_ir_reg<4, 5>(jac, warp);
+    if (rpt <= 8) return pick_ir_reg<8, 5>(jac, warp);
+  } else if (wmax <= 8) {
+    if (rpt <= 1) return pick_ir_reg<1, 8>(jac, warp);
+    if (rpt <= 2) return pick_ir_reg<2, 8>(jac, warp);
+    if (rpt <= 4) return pick_ir_reg<4, 8>(jac, warp);
+  }
+  return nullptr;
+}
+
 // Block size a class runs with before (or without) autotuning.
 int default_threads(int c) { return c <= 1 ? 32 : (c <= 4 ? 64 : 128); }
 
@@ -669,6 +930,7 @@ struct Batch {
   void* ell_val = nullptr;
   float* ell_val32 = nullptr;  // FP64 batches: FP32 copy for refinement
   unsigned int* next = nullptr;  // one counter per class
+  BatchIo* io = nullptr;
   gk_batch_status* st = nullptr;
   double* xtune = nullptr;
   int threads[3][2][kBatchClasses] = {};  // [kind][jacobi][class]; 0 = default
@@ -698,7 +960,11 @@ int plan_class(const Batch& B, int kind, int jac, int c, int threads, ClassPlan*
   p->threads = threads;
   const int elk = kind == GK_IR_CG ? 8 : static_cast<int>(el);
   p->smem = batch_red_offset(kind, jac != 0, elk, k.nmax) + 16 * static_cast<size_t>(threads) + 16;
-  p->fn = pick_kernel(B.dtype, kind, jac != 0, threads);
+  p->fn = kind == GK_IR_CG ? pick_ir_reg(k.nmax, k.wmax, jac != 0, threads) : nullptr;
+  if (p->fn)
+    p->smem = (static_cast<size_t>(kIrRegRowBytes) * k.nmax + 15) / 16 * 16 + 16 * static_cast<size_t>(threads) + 16;
+  else
+    p->fn = pick_kernel(B.dtype, kind, jac != 0, threads);
   int smem_max = 0;
   GK_TRY_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, B.device));
   if (p->smem + 64 > static_cast<size_t>(smem_max))
@@ -712,7 +978,7 @@ int plan_class(const Batch& B, int kind, int jac, int c, int threads, ClassPlan*
   return GK_OK;
 }
 
-BatchArgs class_args(const Batch& B, const gk_criteria& c, const double* b, double* x, int cl) {
+BatchArgs class_args(const Batch& B, const gk_criteria& c, int cl) {
   BatchArgs a;
   a.sys_ptr = B.sys_ptr;
   a.order = B.order;
@@ -721,8 +987,9 @@ BatchArgs class_args(const Batch& B, const gk_criteria& c, const double* b, doub
   a.ell_col = B.ell_col;
   a.ell_val = B.ell_val;
   a.ell_val32 = B.ell_val32;
-  a.b = b;
-  a.x = x;
+  a.io = B.io;
+  a.b = nullptr;
+  a.x = nullptr;
   a.st = B.st;
   a.next = B.next + cl;
   a.max_iters = c.max_iters;
@@ -748,7 +1015,7 @@ void batch_release(Batch* B) {
   cudaSetDevice(B->device);
   if (B->exec) cudaGraphExecDestroy(B->exec);
   void* ptrs[] = {B->sys_ptr, B->order,  B->ell_off, B->ell_w, B->ell_col, B->ell_val,
-                  B->ell_val32, B->next, B->st,     B->xtune};
+                  B->ell_val32, B->next, B->st,     B->xtune, B->io};
   for (void* p : ptrs) dfree(p);
   cudaSetDevice(prev);
   delete B;
@@ -857,6 +1124,7 @@ extern "C" int gk_batch_create(int64_t n_sys, const int64_t* sys_ptr, int64_t nn
   GK_TRY(dalloc_n(&B->sys_ptr, sp32.size(), by));
   GK_TRY(dalloc_n(&B->order, order.size(), by));
   GK_TRY(dalloc_n(&B->next, kBatchClasses, by));
+  GK_TRY(dalloc_n(&B->io, 1, by));
   GK_TRY(dalloc_n(&B->st, static_cast<size_t>(n_sys), by));
   GK_TRY_CUDA(cudaMemcpyAsync(B->sys_ptr, sp32.data(), sizeof(int32_t) * sp32.size(), cudaMemcpyHostToDevice, s));
   GK_TRY_CUDA(cudaMemcpyAsync(B->order, order.data(), sizeof(int32_t) * order.size(), cudaMemcpyHostToDevice, s));
@@ -911,6 +1179,8 @@ extern "C" int gk_batch_create(int64_t n_sys, const int64_t* sys_ptr, int64_t nn
     if (total > INT32_MAX - 16) return set_error(GK_ERR_UNSUPPORTED, "gk_batch_create: ELL storage exceeds 2^31");
   }
   eo[n_sys] = static_cast<int32_t>(total);
+  for (BatchClass& cl : B->cls)
+    for (int k = cl.k0; k < cl.k0 + cl.count; ++k) cl.wmax = std::max(cl.wmax, ew[static_cast<size_t>(order[k])]);
   B->ell_entries = total;
   GK_TRY(dalloc_n(&B->ell_off, eo.size(), by));
   GK_TRY(dalloc_n(&B->ell_w, ew.size(), by));
@@ -952,8 +1222,6 @@ extern "C" int gk_batch_solve(gk_batch h, int32_t kind, int32_t jacobi, const gk
     memset(key, 0, sizeof(key));
     key[0] = static_cast<uint64_t>(kind);
     key[1] = static_cast<uint64_t>(jacobi != 0);
-    key[2] = reinterpret_cast<uint64_t>(b);
-    key[3] = reinterpret_cast<uint64_t>(x);
     key[4] = static_cast<uint64_t>(crit->max_iters);
     memcpy(&key[5], &crit->reduction_factor, sizeof(double));
     key[6] = static_cast<uint64_t>(crit->rel_to_b);
@@ -970,7 +1238,7 @@ extern "C" int gk_batch_solve(gk_batch h, int32_t kind, int32_t jacobi, const gk
       for (int c = 0; c < kBatchClasses && rc == GK_OK; ++c) {
         if (!B->cls[c].count) continue;
         rc = plan_class(*B, kind, jacobi, c, class_threads(*B, kind, jacobi, c), &plan[c]);
-        args[c] = class_args(*B, *crit, static_cast<const double*>(b), static_cast<double*>(x), c);
+        args[c] = class_args(*B, *crit, c);
       }
       if (rc != GK_OK) break;
       cudaStream_t cs = nullptr;
@@ -995,7 +1263,9 @@ extern "C" int gk_batch_solve(gk_batch h, int32_t kind, int32_t jacobi, const gk
       }
       memcpy(B->key, key, sizeof(key));
     }
-    cudaError_t e = cudaGraphLaunch(B->exec, s);
+    const BatchIo io = {static_cast<const double*>(b), static_cast<double*>(x)};
+    cudaError_t e = cudaMemcpyAsync(B->io, &io, sizeof(io), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaGraphLaunch(B->exec, s);
     if (e != cudaSuccess) {
       rc = cuda_error(e, "gk_batch_solve: graph launch");
       break;
@@ -1049,7 +1319,9 @@ extern "C" int gk_batch_autotune(gk_batch h, int32_t kind, int32_t jacobi, const
   int chosen[kBatchClasses] = {};
   do {
     if (!B->xtune && (rc = dalloc_n(&B->xtune, static_cast<size_t>(B->n_rows), &B->device_bytes))) break;
-    cudaError_t e = cudaEventCreate(&e0);
+    const BatchIo io = {static_cast<const double*>(b), B->xtune};
+    cudaError_t e = cudaMemcpyAsync(B->io, &io, sizeof(io), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e != cudaSuccess) {
       rc = cuda_error(e, "events");
@@ -1059,7 +1331,7 @@ extern "C" int gk_batch_autotune(gk_batch h, int32_t kind, int32_t jacobi, const
       if (times_ms)
         for (int j = 0; j < 4; ++j) times_ms[c * 4 + j] = -1.0;
       if (!B->cls[c].count) continue;
-      BatchArgs a = class_args(*B, *crit, static_cast<const double*>(b), B->xtune, c);
+      BatchArgs a = class_args(*B, *crit, c);
       a.st = nullptr;
       float best_ms = 0.0f;
       for (int j = 0; j < 4 && rc == GK_OK; ++j) {
