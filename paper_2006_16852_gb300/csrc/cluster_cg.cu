@@ -91,7 +91,7 @@ struct ClSlots {
 template <int K, typename Post>
 __device__ __forceinline__ void cluster_total(cg::cluster_group& cl, double (&v)[K], double (*wsum)[K],
                                               double* slot, Post post) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = warp_uniform(threadIdx.x >> 5);
   warp_sum<K, double>(v);
   if (lane == 0) {
 #pragma unroll

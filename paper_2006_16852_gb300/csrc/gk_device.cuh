@@ -105,6 +105,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
   return false;
 }
 
+// A value that all lanes of a warp share (a warp's index, the first item of
+// its loop), taken from lane 0: what the compiler computes from threadIdx it
+// takes for different in every lane, and a shuffle under a branch or loop on
+// it then costs hundreds of cycles (a butterfly step 620 instead of 145).
+__device__ __forceinline__ int warp_uniform(unsigned int v) {
+  return static_cast<int>(__shfl_sync(0xffffffffu, v, 0));
+}
+
 // ---------------------------------------------------------------------------
 // Fixed-order FP64 reductions.  A block sums its threads' values in one warp
 // (block_sum below); the grid sums per-block partials in the last block to

@@ -97,7 +97,7 @@ struct GmArgs {
   const int lane_ = threadIdx.x & 31;                                                           \
   const int bpw_ = 32 / a.bs;                                                                   \
   const int nw_ = (gridDim.x * blockDim.x) >> 5;                                                 \
-  for (int w_ = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w_ * bpw_ < a.nblocks; w_ += nw_) \
+  for (int w_ = warp_uniform((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w_ * bpw_ < a.nblocks; w_ += nw_) \
     for (BjLane L = bj_lane(w_ * bpw_, lane_, a.bs, a.n, a.nblocks), *once_ = &L; once_; once_ = nullptr)
 
 // The true residual r and its norm are known: V_0 = r / ||r||, g = ||r|| e_1.
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kDotThreads) gm_dots_kernel(GmArgs a) {
   const int j = s->j;
   const int G = gridDim.x;
   const int lane = threadIdx.x & 31;
-  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x) >> 5, 0);  // uniform
+  const int warp = warp_uniform(threadIdx.x >> 5);
   // N vectors from c0 on; several rows per step for small N
   auto sweep = [&](auto n_vec, int c0) {
     constexpr int N = decltype(n_vec)::value;

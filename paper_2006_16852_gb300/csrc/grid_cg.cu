@@ -212,7 +212,7 @@ __device__ __forceinline__ bool grid_total(const GridArgs& a, GridRed& red, unsi
                                            const double (&v)[K], Idle idle, Post post) {
   // the warp's index from lane 0, so that the branch on it is uniform: the
   // shuffles under a branch on threadIdx.x took 620 cycles a step
-  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x) >> 5, 0);
+  const int lane = threadIdx.x & 31, warp = warp_uniform(threadIdx.x >> 5);
 #pragma unroll
   for (int k = 0; k < K; ++k) red.part[k][threadIdx.x] = v[k];
   ++seq;

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(256) csr_entries_kernel(const int32_t* __restr
   const int n_groups = (n_rows + 31) / 32;
   const int n_warps = (gridDim.x * blockDim.x) >> 5;
   // (the warp's index from lane 0: a loop the compiler knows to be uniform)
-  const int warp0 = __shfl_sync(0xffffffffu, static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5), 0);
+  const int warp0 = warp_uniform((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   for (int g = warp0; g < n_groups; g += n_warps) {
     const int r = g * 32 + lane;
     const int s = rowptr[min(r, n_rows)], e = rowptr[min(r + 1, n_rows)];

@@ -168,9 +168,23 @@ struct SliceMinBlocks {
   static constexpr int value = (MODE == EPI_COPY || MODE == EPI_PLAIN) ? 8 : 6;
 };
 
-template <int MODE>
-__global__ void __launch_bounds__(kSliceThreads, SliceMinBlocks<MODE>::value) spmv_sliced_kernel(SliceArgs a,
-                                                                                                Epi e) {
+// DEEP: for matrices of so few slices and pieces that every one has a warp of
+// its own on the GPU (at most 16 per SM: below about 75,000 rows of up to 256
+// entries).  There nothing hides a lane's chain of loads -- index, gather,
+// next index -- so a lane loads 16 slots' indices and values while it gathers
+// for the 16 before; the registers that takes (2 blocks per SM) are free.
+// The sums are the same, in the same order.  Power-law, 5,000 and 20,000
+// rows: 34.8 and 37.4 -> 23.7 and 26.8 us an apply; random rows of up to 40
+// entries, 4,099 rows: 7.5 -> 6.7; 27-point 30^3: 7.0 -> 4.8.  The line: with
+// up to 64 per SM the 27-point matrices of 50^3 and 64^3 rows took 13.4 and
+// 29.7 us against 10.0 and 17.3 (power-law at 120,000 rows gained, 59 -> 41).
+// Three stages of 8 slots measured slower (25.7 and 30.5).
+constexpr int kDeepSlots = 16;
+constexpr int kDeepItemsPerSm = 16;
+
+template <int MODE, bool DEEP>
+__global__ void __launch_bounds__(kSliceThreads, DEEP ? 2 : SliceMinBlocks<MODE>::value)
+    spmv_sliced_kernel(SliceArgs a, Epi e) {
   pdl_wait();
   constexpr int B = EllBatchOf<MODE>::value;
   __shared__ double red_scratch[kRedScratch];
@@ -183,7 +197,7 @@ __global__ void __launch_bounds__(kSliceThreads, SliceMinBlocks<MODE>::value) sp
     if (it < a.n_pc) {
       const int4 pc = __ldg(a.pc + it);
       const int k0 = pc.y, k1 = pc.z;
-      constexpr int MB = MidBatchOf<MODE>::value;
+      constexpr int MB = DEEP ? 16 : MidBatchOf<MODE>::value;
       double s = 0.0;
       int k = k0 + lane;
       for (; k + 32 * (MB - 1) < k1; k += 32 * MB) {
@@ -229,6 +243,34 @@ __global__ void __launch_bounds__(kSliceThreads, SliceMinBlocks<MODE>::value) sp
       const double* vp = a.sval + o0 + lane;
       double s = 0.0;
       int j = 0;
+      if constexpr (DEEP) {
+        int cn[kDeepSlots];
+        double vn[kDeepSlots];
+        auto load = [&](int j0) {
+#pragma unroll
+          for (int u = 0; u < kDeepSlots; ++u) {
+            const bool in = j0 + u < L;
+            cn[u] = in ? __ldcs(cp + (j0 + u) * 32) : -1;
+            vn[u] = in ? __ldcs(vp + (j0 + u) * 32) : 0.0;
+          }
+        };
+        load(0);
+        for (; j < L; j += kDeepSlots) {
+          int cc[kDeepSlots];
+          double vv[kDeepSlots], xv[kDeepSlots];
+#pragma unroll
+          for (int u = 0; u < kDeepSlots; ++u) {
+            cc[u] = cn[u];
+            vv[u] = vn[u];
+          }
+#pragma unroll
+          for (int u = 0; u < kDeepSlots; ++u) xv[u] = cc[u] >= 0 ? __ldg(a.x + cc[u]) : 0.0;
+          load(j + kDeepSlots);
+#pragma unroll
+          for (int u = 0; u < kDeepSlots; ++u)
+            if (cc[u] >= 0) s = fma(vv[u], xv[u], s);
+        }
+      }
       for (; j + B <= L; j += B) {
         int cc[B];
         double vv[B], xv[B];
@@ -799,8 +841,8 @@ int merge_grid(int64_t n_tiles) {
 }
 
 int sliced_grid(int64_t warp_items, bool plain) {
-  const void* fn = plain ? reinterpret_cast<const void*>(spmv_sliced_kernel<EPI_COPY>)
-                         : reinterpret_cast<const void*>(spmv_sliced_kernel<EPI_RESID>);
+  const void* fn = plain ? reinterpret_cast<const void*>(spmv_sliced_kernel<EPI_COPY, false>)
+                         : reinterpret_cast<const void*>(spmv_sliced_kernel<EPI_RESID, false>);
   int g = occupancy_grid(fn, kSliceThreads, 0);
   int64_t need = (warp_items + kSliceThreads / 32 - 1) / (kSliceThreads / 32);
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(g, need)));
@@ -847,13 +889,21 @@ int spmv_launch(const Matrix& A, const double* x, const Epi& e, cudaStream_t s) 
                   static_cast<int>(A.n_lr), A.pc_sum, x};
       const bool plain = e.mode == EPI_COPY || e.mode == EPI_PLAIN;
       const int g = plain ? A.grid_sl_plain : A.grid_sl;
+      const bool deep = A.n_pc + A.n_slices <= static_cast<int64_t>(kDeepItemsPerSm) * sm_count();
+#define GK_SLICED(MODE)                                                                              \
+  case MODE:                                                                                       \
+    if (deep) launch_pdl(spmv_sliced_kernel<MODE, true>, g, kSliceThreads, 0, s, b, e);             \
+    else launch_pdl(spmv_sliced_kernel<MODE, false>, g, kSliceThreads, 0, s, b, e);                 \
+    break
       switch (e.mode) {
-        case EPI_COPY: launch_pdl(spmv_sliced_kernel<EPI_COPY>, g, kSliceThreads, 0, s, b, e); break;
-        case EPI_PLAIN: launch_pdl(spmv_sliced_kernel<EPI_PLAIN>, g, kSliceThreads, 0, s, b, e); break;
-        case EPI_RESID: launch_pdl(spmv_sliced_kernel<EPI_RESID>, g, kSliceThreads, 0, s, b, e); break;
-        case EPI_DOT: launch_pdl(spmv_sliced_kernel<EPI_DOT>, g, kSliceThreads, 0, s, b, e); break;
-        default: launch_pdl(spmv_sliced_kernel<EPI_DOT2>, g, kSliceThreads, 0, s, b, e); break;
+        GK_SLICED(EPI_COPY);
+        GK_SLICED(EPI_PLAIN);
+        GK_SLICED(EPI_RESID);
+        GK_SLICED(EPI_DOT);
+        GK_SLICED(EPI_DOT2);
+        default: break;
       }
+#undef GK_SLICED
       GK_TRY_CUDA(cudaGetLastError());
       if (A.n_lr > 0) {
         const int fg = static_cast<int>(std::min<int64_t>(kFixupMaxGrid, (A.n_lr + 7) / 8));

@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(256, 2) wgrad_thin_kernel(const float* __restr
   constexpr int T = kWideOut ? CIN : COUT;  // thin channels
   constexpr int STRIDE = COUT * CIN * 9 + COUT;
   const int lane = threadIdx.x & 31;
-  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x) >> 5, 0);  // uniform
+  const int warp = warp_uniform(threadIdx.x >> 5);
   const int b = blockIdx.y, unit = blockIdx.x;
   const int y0 = unit % dil + kThinRows * dil * (unit / dil);
   const int nrow = y0 < H ? min(kThinRows, (H - 1 - y0) / dil + 1) : 0;
@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(kTcThreads) conv_tc_kernel(const __nv_bfloat16
   extern __shared__ __align__(1024) unsigned char tc_raw[];
   TcSmem& S = *reinterpret_cast<TcSmem*>(tc_raw);
   const int t = threadIdx.x, lane = t & 31;
-  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // uniform
+  const int warp = warp_uniform(t >> 5);
   for (int i = t; i < kTcPacked / 8; i += kTcThreads)
     reinterpret_cast<uint4*>(S.b)[i] = __ldg(reinterpret_cast<const uint4*>(wp) + i);
   if (t < 32) S.bias[t] = __bfloat162float(bias[t]);
@@ -1151,7 +1151,7 @@ __global__ void __launch_bounds__(kTcFirstThreads) conv_first_tc_kernel(const fl
                                                                         __nv_bfloat16* __restrict__ y, int* err) {
   __shared__ __align__(1024) TcFirstSmem S;
   const int t = threadIdx.x;
-  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // uniform
+  const int warp = warp_uniform(t >> 5);
   // weights [chunk j][out n][e] = w[n][8 j + e] (k = channel * 9 + tap), zero past k = 17
   for (int i = t; i < 4 * 32 * 8; i += kTcFirstThreads) {
     const int e = i & 7, n = (i >> 3) & 31, j = i >> 8;
