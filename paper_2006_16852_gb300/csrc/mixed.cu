@@ -250,9 +250,20 @@ struct Ell32 {
   unsigned int* counter;
 };
 
+// Bound by latency before bandwidth: a row is two dependent loads (column,
+// then x) however many slots it has, as long as the slots are loaded
+// together.  Eight at a time, those past K skipped under a predicate: the
+// seven slots of a 7-point operator are one such pair (batches of 4 with the
+// rest one by one were four).  That takes 40 registers, so six blocks per SM,
+// and the grid is no larger than what is resident.  7-point 128^3: 28 us per
+// SpMV, 117 MB of matrix at 4.2 TB/s; refinement of it to 1e-12 31.9 ->
+// 25.8 ms (batches of 4 with predicates: 28.2; five blocks per SM: the same).
+constexpr int kEll32Batch = 8;
+constexpr int kEll32Blocks = 6;
+
 template <bool TAIL, bool DOT>
-__global__ void __launch_bounds__(kIrThreads, 8) ir_spmv_ell_kernel(Ell32 a, const float* __restrict__ x,
-                                                                     float* __restrict__ y) {
+__global__ void __launch_bounds__(kIrThreads, kEll32Blocks)
+    ir_spmv_ell_kernel(Ell32 a, const float* __restrict__ x, float* __restrict__ y) {
   pdl_wait();
   __shared__ float scratch[kRedScratch];
   if (a.ist->done) return;
@@ -261,30 +272,27 @@ __global__ void __launch_bounds__(kIrThreads, 8) ir_spmv_ell_kernel(Ell32 a, con
   for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < a.n; row += stride) {
     const int32_t* cp = a.col + row;
     const float* vp = a.val + row;
+    const float xr = DOT ? x[row] : 0.0f;
     float s = 0.0f;
-    int j = 0;
-    for (; j + 4 <= a.K; j += 4) {
-      int cc[4];
-      float vv[4], xv[4];
+    for (int j = 0; j < a.K; j += kEll32Batch) {
+      int cc[kEll32Batch];
+      float vv[kEll32Batch], xv[kEll32Batch];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) cc[u] = __ldcs(cp + (j + u) * a.ld);
+      for (int u = 0; u < kEll32Batch; ++u) cc[u] = j + u < a.K ? __ldcs(cp + (j + u) * a.ld) : -1;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) vv[u] = __ldcs(vp + (j + u) * a.ld);
+      for (int u = 0; u < kEll32Batch; ++u) vv[u] = j + u < a.K ? __ldcs(vp + (j + u) * a.ld) : 0.0f;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) xv[u] = cc[u] >= 0 ? __ldg(x + cc[u]) : 0.0f;
+      for (int u = 0; u < kEll32Batch; ++u) xv[u] = cc[u] >= 0 ? __ldg(x + cc[u]) : 0.0f;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) s = fmaf(vv[u], xv[u], s);
-    }
-    for (; j < a.K; ++j) {
-      const int c = __ldcs(cp + j * a.ld);
-      if (c >= 0) s = fmaf(__ldcs(vp + j * a.ld), __ldg(x + c), s);
+      for (int u = 0; u < kEll32Batch; ++u)
+        if (cc[u] >= 0) s = fmaf(vv[u], xv[u], s);
     }
     if (TAIL) {
       const int t = __ldg(a.tail_slot + row);
       if (t >= 0) s += __ldcg(a.tail_sum + t);
     }
     y[row] = s;
-    if (DOT) a0 = fmaf(x[row], s, a0);
+    if (DOT) a0 = fmaf(xr, s, a0);
   }
   if (DOT) {
     float v[1] = {a0}, out[1];
@@ -334,10 +342,11 @@ __global__ void __launch_bounds__(kIrThreads, 8) ir_spmv_csr_kernel(const int32_
 #define IR_FOR_ROWS(i) for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x)
 #define IR_FOR_BLOCK_LANES(L)                                                                        \
   const int lane_ = threadIdx.x & 31;                                                                \
-  const int bpw_ = 32 / a.bs;                                                                        \
+  const int bs_ = BS > 0 ? BS : a.bs;                                                                \
+  const int bpw_ = 32 / bs_;                                                                         \
   const int nw_ = (gridDim.x * blockDim.x) >> 5;                                                      \
   for (int w_ = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w_ * bpw_ < a.nblocks; w_ += nw_)      \
-    for (BjLane L = bj_lane(w_ * bpw_, lane_, a.bs, a.n, a.nblocks), *once_ = &L; once_; once_ = nullptr)
+    for (BjLane L = bj_lane(w_ * bpw_, lane_, bs_, a.n, a.nblocks), *once_ = &L; once_; once_ = nullptr)
 
 // r = r64 / ||r64||, d = 0, z = M^{-1} r, p = z, rho = r.z, rr0 = r.r.
 template <int PK, int BS>
@@ -397,13 +406,22 @@ struct DInDirection {
   static constexpr bool value = PK == PREC_BLOCK;
 };
 
+// Resident blocks per SM, also the grid: the rows of a block of 16 or 32 in
+// registers leave room for five or four, and blocks beyond those would run as
+// a second, partly empty wave (bs = 16 on 7-point 100^3: refinement 17.7 ->
+// 13.1 ms together with the other two kernels).  Two sets of blocks in flight per warp instead
+// of one, at five resident blocks, measured the same at bs = 8 (four at three
+// 5 % slower).
+template <int PK, int BS>
+constexpr int kUpdateBlocks = PK != PREC_BLOCK ? 8 : BS == 32 ? 4 : BS == 16 ? 5 : BS == 0 ? 6 : 8;
+
 // [d += alpha p;] r -= alpha q; z = M^{-1} r; (r.z, r.r); inner criteria.
 // When the direction kernel updates d, it must know whether this
 // iteration's update ran: block 0 first records the iteration count the
 // direction kernel last caught up with (before any early return), and the
 // finalize raises the count past it only if the update runs.
 template <int PK, int BS>
-__global__ void __launch_bounds__(kIrThreads) ir_update_kernel(IrArgs a, IrData d) {
+__global__ void __launch_bounds__(kIrThreads, kUpdateBlocks<PK, BS>) ir_update_kernel(IrArgs a, IrData d) {
   pdl_wait();
   __shared__ float scratch[kRedScratch];
   if (blockIdx.x == 0 && threadIdx.x == 0) d.ist->d_it = d.ist->it;
@@ -453,6 +471,9 @@ __global__ void __launch_bounds__(kIrThreads) ir_update_kernel(IrArgs a, IrData 
 
 // [d += alpha p if this iteration's update ran (it past d_it),] then
 // p = z + beta p unless the inner solve is done; re-arms the inner loop.
+// Four rows per thread with 16-byte accesses (each vector is an allocation of
+// its own); at 128^3 the vectors are in L2 and it takes 6.4 us for 42 MB
+// (refinement 25.8 -> 24.9 ms against one row per thread).
 template <int PK>
 __global__ void __launch_bounds__(kIrThreads) ir_direction_kernel(IrArgs a, IrData d) {
   pdl_wait();
@@ -465,16 +486,29 @@ __global__ void __launch_bounds__(kIrThreads) ir_direction_kernel(IrArgs a, IrDa
   }
   if (!dup && !pup) return;
   const float alpha = static_cast<float>(s->alpha), beta = static_cast<float>(s->beta);
-  IR_FOR_ROWS(i) {
+  const float* zp = PK == PREC_BLOCK ? d.z : d.r;
+  const int n4 = a.n >> 2, t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  for (int i = t; i < n4; i += nt) {
+    const float4 pv = reinterpret_cast<const float4*>(d.p)[i];
+    if (pup) {
+      float4 zv = reinterpret_cast<const float4*>(zp)[i];
+      if (PK == PREC_SCALAR) {
+        const float4 iv = reinterpret_cast<const float4*>(d.dinv)[i];
+        zv = make_float4(iv.x * zv.x, iv.y * zv.y, iv.z * zv.z, iv.w * zv.w);
+      }
+      reinterpret_cast<float4*>(d.p)[i] = make_float4(fmaf(beta, pv.x, zv.x), fmaf(beta, pv.y, zv.y),
+                                                      fmaf(beta, pv.z, zv.z), fmaf(beta, pv.w, zv.w));
+    }
+    if (dup) {
+      const float4 dv = reinterpret_cast<const float4*>(d.d)[i];
+      reinterpret_cast<float4*>(d.d)[i] = make_float4(fmaf(alpha, pv.x, dv.x), fmaf(alpha, pv.y, dv.y),
+                                                      fmaf(alpha, pv.z, dv.z), fmaf(alpha, pv.w, dv.w));
+    }
+  }
+  for (int i = 4 * n4 + t; i < a.n; i += nt) {
     const float pv = d.p[i];
     if (dup) d.d[i] = fmaf(alpha, pv, d.d[i]);
-    if (pup) {
-      float zv;
-      if (PK == PREC_BLOCK) zv = d.z[i];
-      else if (PK == PREC_SCALAR) zv = d.dinv[i] * d.r[i];
-      else zv = d.r[i];
-      d.p[i] = fmaf(beta, pv, zv);
-    }
+    if (pup) d.p[i] = fmaf(beta, pv, PK == PREC_SCALAR ? d.dinv[i] * zp[i] : zp[i]);
   }
 }
 
@@ -552,14 +586,15 @@ int ir_spmv(const Solver& S, const IrData& d, const IrArgs& a, cudaStream_t s) {
   const Matrix& A = *S.A;
   if (d.fmt == GK_ELL) {
     const bool tail = A.format == GK_HYB && A.m_tail > 0;
+    const int grid = std::min(d.grid, kEll32Blocks * sm_count());
     const Ell32 e32{A.ell_col, d.ell_val32, A.ld, static_cast<int>(A.K), a.n, A.tail_slot, d.tail_sum32,
                     d.ist, d.partials, d.counter};
     if (tail) {
       launch_csr32<false>(d.tail_lpr, d.grid, s, A.tail_rowptr, A.tail_col, d.tail_val32,
                           static_cast<int>(A.m_tail), d, d.p, d.tail_sum32);
-      launch_pdl(ir_spmv_ell_kernel<true, true>, d.grid, kIrThreads, 0, s, e32, d.p, d.q);
+      launch_pdl(ir_spmv_ell_kernel<true, true>, grid, kIrThreads, 0, s, e32, d.p, d.q);
     } else {
-      launch_pdl(ir_spmv_ell_kernel<false, true>, d.grid, kIrThreads, 0, s, e32, d.p, d.q);
+      launch_pdl(ir_spmv_ell_kernel<false, true>, grid, kIrThreads, 0, s, e32, d.p, d.q);
     }
   } else {
     launch_csr32<true>(d.lpr, d.grid, s, A.rowptr, A.col, d.val32, a.n, d, d.p, d.q);
@@ -596,7 +631,11 @@ int ir_enqueue_start(const Solver& S, const IrData& d, const IrArgs& a, cudaStre
 int ir_enqueue_inner(const Solver& S, const IrData& d, const IrArgs& a, cudaStream_t s) {
   GK_TRY(ir_spmv(S, d, a, s));
   if (S.pk == PREC_BLOCK) {
-    IR_LAUNCH_BS(ir_update_kernel, a.bs, d.grid, s, a, d);
+    const int blocks = a.bs == 4 || a.bs == 8 ? kUpdateBlocks<PREC_BLOCK, 8>
+                       : a.bs == 16           ? kUpdateBlocks<PREC_BLOCK, 16>
+                       : a.bs == 32           ? kUpdateBlocks<PREC_BLOCK, 32>
+                                              : kUpdateBlocks<PREC_BLOCK, 0>;
+    IR_LAUNCH_BS(ir_update_kernel, a.bs, std::min(d.grid, blocks * sm_count()), s, a, d);
     launch_pdl(ir_direction_kernel<PREC_BLOCK>, d.grid, kIrThreads, 0, s, a, d);
   } else if (S.pk == PREC_SCALAR) {
     launch_pdl(ir_update_kernel<PREC_SCALAR, 0>, d.grid, kIrThreads, 0, s, a, d);
