@@ -64,7 +64,7 @@ struct BatchArgs {
   const void* ell_val;      // values in the solve precision
   const float* ell_val32;   // FP32 copy of FP64 values (refinement inner solves)
   const BatchIo* io;
-  const double* b;  // io's, read by each block
+  const double* b;  // io's, for batch_ir_reg_kernel, which keeps them in registers
   double* x;
   gk_batch_status* st;
   unsigned int* next;  // this class's counter
@@ -102,6 +102,15 @@ __device__ __forceinline__ void reduce(T (&v)[K], T* red, double* sc, double (&o
 #pragma unroll
     for (int s = 0; s < S; ++s) out[s] = sc[s];
   }
+}
+
+// The vectors where they are used, once per system: kept in a kernel's copy of
+// its arguments they cost FP32 CG 2.13 -> 2.66 ms on 10,000 systems.
+__device__ __forceinline__ const double* io_b(const BatchArgs& a) {
+  return reinterpret_cast<const double*>(__ldg(reinterpret_cast<const unsigned long long*>(&a.io->b)));
+}
+__device__ __forceinline__ double* io_x(const BatchArgs& a) {
+  return reinterpret_cast<double*>(__ldg(reinterpret_cast<const unsigned long long*>(&a.io->x)));
 }
 
 // One system's matrix: n rows, ELL width w, entry (k, i) at k * n + i.
@@ -156,7 +165,7 @@ __device__ __forceinline__ void sys_jacobi(const SysMat<T>& m, T* D) {
 template <typename T>
 __device__ __forceinline__ void sys_finish(const BatchArgs& a, const T* X, int sys, int r0, int n, long long it,
                                            int stop, double rnorm, double ref) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) a.x[r0 + i] = static_cast<double>(X[i]);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) io_x(a)[r0 + i] = static_cast<double>(X[i]);
   if (threadIdx.x == 0 && a.st) {
     a.st[sys].iters = static_cast<int32_t>(it);
     a.st[sys].stop_reason = stop;
@@ -173,7 +182,7 @@ __device__ __forceinline__ void sys_start(const BatchArgs& a, const SysMat<T>& m
   sys_spmv<T>(m, X, Q);
   T s2[2] = {T(0), T(0)};
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const T bi = static_cast<T>(a.b[r0 + i]);
+    const T bi = static_cast<T>(io_b(a)[r0 + i]);
     const T ri = bi - Q[i];
     R[i] = ri;
     if (RH) RH[i] = ri;
@@ -199,7 +208,7 @@ __device__ void cg_system(const BatchArgs& a, T* V, T* red, double* sc, int sys,
   const SysMat<T> m = sys_mat<T>(a, sys, n);
   const int nm = a.nmax;
   T *X = V, *R = V + nm, *P = V + 2 * nm, *Q = V + 3 * nm, *D = V + 4 * nm;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) X[i] = static_cast<T>(a.x[r0 + i]);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) X[i] = static_cast<T>(io_x(a)[r0 + i]);
   if (JAC) sys_jacobi<T>(m, D);
   __syncthreads();
   double rnorm, ref;
@@ -281,7 +290,7 @@ __device__ void bicg_system(const BatchArgs& a, T* V, T* red, double* sc, int sy
   const T* PH = JAC ? H : P;  // p^ = M^-1 p
   const T* SH = JAC ? H : R;  // s^ = M^-1 s (s lives in R)
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    X[i] = static_cast<T>(a.x[r0 + i]);
+    X[i] = static_cast<T>(io_x(a)[r0 + i]);
     P[i] = T(0);
   }
   if (JAC) sys_jacobi<T>(m, D);
@@ -429,7 +438,7 @@ __device__ void ir_system(const BatchArgs& a, unsigned char* smem, double* redd,
   float *P = R + nm, *Q = R + 2 * nm, *DX = R + 3 * nm, *D = R + 4 * nm;
   float* redf = reinterpret_cast<float*>(redd);
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    X[i] = a.x[r0 + i];
+    X[i] = io_x(a)[r0 + i];
     if (JAC) {
       double d = 0.0;
       for (int k = 0; k < m64.w; ++k)
@@ -450,7 +459,7 @@ __device__ void ir_system(const BatchArgs& a, unsigned char* smem, double* redd,
     sys_spmv<double>(m64, X, R64);
     double s2[2] = {0.0, 0.0};
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const double bi = a.b[r0 + i];
+      const double bi = io_b(a)[r0 + i];
       const double ri = bi - R64[i];
       R64[i] = ri;
       s2[0] = fma(ri, ri, s2[0]);
@@ -558,7 +567,7 @@ __device__ void ir_system(const BatchArgs& a, unsigned char* smem, double* redd,
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) a.x[r0 + i] = X[i];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) io_x(a)[r0 + i] = X[i];
   if (threadIdx.x == 0 && a.st) {
     a.st[sys].iters = static_cast<int32_t>(k_total);
     a.st[sys].stop_reason = stop;
@@ -596,8 +605,7 @@ __device__ __forceinline__ void sum32(float (&v)[K], float (*ws)[2][8], int& par
 // shared memory and has three barriers; ir_system reads the matrix from
 // L1/L2 and five vectors from shared memory in every iteration, with eight
 // barriers, and its latency is what 10,000 systems of 36 to 1,024 rows wait
-// for: 5.76 -> 3.58 ms to 1e-12 with
-// one graph for all vectors (above).
+// for: 5.76 -> 3.58 ms to 1e-12, with one graph for all vectors (above).
 template <int RPT, int W, bool JAC, bool WARP>
 __device__ void ir_system_reg(const BatchArgs& a, unsigned char* smem, double* redd, double* sc, float (*ws)[2][8],
                               int sys, int r0, int n) {
@@ -785,8 +793,6 @@ __global__ void __launch_bounds__(256) batch_kernel(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char bsm[];
   __shared__ double s_sc[4];
   __shared__ int s_k;
-  a.b = a.io->b;
-  a.x = a.io->x;
   T* V = reinterpret_cast<T*>(bsm);
   unsigned char* redp = bsm + batch_red_offset(KIND, JAC, static_cast<int>(sizeof(T)), a.nmax);
   T* red = reinterpret_cast<T*>(redp);
