@@ -149,6 +149,7 @@ struct SliceArgs {
   const int32_t* scol;
   const double* sval;
   int n_sell, n_slices;
+  int n_split;            // slices (the first ones) taken by four warps each; SL_SPLIT only
   const int4* pc;        // pieces of the long rows: {row, k0, k1, slot}
   int n_pc;
   const int32_t* lr_row;  // rows of several pieces and their slots
@@ -182,20 +183,71 @@ struct SliceMinBlocks {
 constexpr int kDeepSlots = 16;
 constexpr int kDeepItemsPerSm = 16;
 
-template <int MODE, bool DEEP>
-__global__ void __launch_bounds__(kSliceThreads, DEEP ? 2 : SliceMinBlocks<MODE>::value)
+// SL_SPLIT: for matrices with a few slices much longer than a warp's share of
+// the work.  Resident warps advance at the same pace, so a warp with a slice
+// of 256 slots is still at it when the others, with about 110 slots each on
+// the power-law matrix, are done, and then runs at the speed of its own chain
+// of loads.  Such a slice is taken by four warps, 8 rows each, whose lanes
+// load 16 slots of a row at once and hand them round by shuffle (the sums and
+// their order stay the same; the FP64 adds of these slices are issued four
+// times, so they are split only where they make up at most an eighth of the
+// work: 8 % there).
+// Power-law of 10^6 rows: 167.9 -> 141.6 us an apply, 1.08x the gather
+// ceiling (back to back 150.6 -> 139.4, with the fused dot 171.4 -> 155.2);
+// 300,000 rows 80 -> 60 us; 120,000 rows 58 -> 38 us.
+enum SliceKind { SL_PLAIN = 0, SL_DEEP = 1, SL_SPLIT = 2 };
+
+// The line: slices of more than 0.6 times a warp's share of all slots, and at
+// least 64.  At 0.3 (and 32) 10^6 rows took 146 us back to back (dot 164), at
+// 0.9 135 (168), at 0.6 138 (154); 120,000 and 300,000 rows are within 6 %.
+constexpr int kSplitMinSlots = 64;
+
+template <int MODE, int KIND>
+__global__ void __launch_bounds__(kSliceThreads, KIND == SL_DEEP ? 2 : SliceMinBlocks<MODE>::value)
     spmv_sliced_kernel(SliceArgs a, Epi e) {
   pdl_wait();
+  constexpr bool DEEP = KIND == SL_DEEP;
   constexpr int B = EllBatchOf<MODE>::value;
   __shared__ double red_scratch[kRedScratch];
   if (epi_skip(e)) return;
   double a0 = 0.0, a1 = 0.0;
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-  const int n_items = a.n_pc + a.n_slices;
-  for (int it = gw; it < n_items; it += nw) {
-    if (it < a.n_pc) {
-      const int4 pc = __ldg(a.pc + it);
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  const int n_quarters = KIND == SL_SPLIT ? 4 * a.n_split : 0;
+  const int n_items = a.n_pc + a.n_slices + (KIND == SL_SPLIT ? 3 * a.n_split : 0);
+  int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (KIND == SL_SPLIT) it = warp_uniform(it);  // a quarter's shuffles are under branches on it
+  for (; it < n_items; it += nw) {
+    if (KIND == SL_SPLIT && it < n_quarters) {
+      // rows 8 (it mod 4) ... of slice it / 4, four lanes a row: a lane loads
+      // every fourth of 16 slots, and all four sum the 16 in slot order
+      // (padding multiplies 0 by -0, which changes no sum)
+      const int c = it >> 2, q = lane & 3, rl = (it & 3) * 8 + (lane >> 2);
+      const int64_t o0 = __ldg(a.off + c);
+      const int L = static_cast<int>((__ldg(a.off + c + 1) - o0) >> 5);
+      const int32_t* cp = a.scol + o0 + rl;
+      const double* vp = a.sval + o0 + rl;
+      double s = 0.0;
+      for (int j = q; j < L + q; j += 16) {
+        int cc[4];
+        double vv[4], xv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const bool in = j + 4 * u < L;
+          cc[u] = in ? __ldcs(cp + (j + 4 * u) * 32) : -1;
+          vv[u] = in ? __ldcs(vp + (j + 4 * u) * 32) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) xv[u] = cc[u] >= 0 ? __ldg(a.x + cc[u]) : -0.0;
+#pragma unroll
+        for (int t = 0; t < 16; ++t)
+          s = fma(__shfl_sync(0xffffffffu, vv[t >> 2], (lane & ~3) | (t & 3)),
+                  __shfl_sync(0xffffffffu, xv[t >> 2], (lane & ~3) | (t & 3)), s);
+      }
+      const int base = c * 32 + rl;
+      if (q == 0 && base < a.n_sell) epi_row_t<MODE>(e, __ldg(a.perm + base), s, a0, a1);
+    } else if (it < n_quarters + a.n_pc) {
+      const int4 pc = __ldg(a.pc + it - n_quarters);
       const int k0 = pc.y, k1 = pc.z;
       constexpr int MB = DEEP ? 16 : MidBatchOf<MODE>::value;
       double s = 0.0;
@@ -235,7 +287,7 @@ __global__ void __launch_bounds__(kSliceThreads, DEEP ? 2 : SliceMinBlocks<MODE>
         else a.pc_sum[pc.w] = s;
       }
     } else {
-      const int c = it - a.n_pc;
+      const int c = it - a.n_pc - (KIND == SL_SPLIT ? 3 * a.n_split : 0);
       const int base = c * 32 + lane;
       const int64_t o0 = __ldg(a.off + c);
       const int L = static_cast<int>((__ldg(a.off + c + 1) - o0) >> 5);
@@ -840,9 +892,24 @@ int merge_grid(int64_t n_tiles) {
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(g, (n_tiles + kMergeWarps - 1) / kMergeWarps)));
 }
 
+static bool sliced_deep(int64_t items) { return items <= static_cast<int64_t>(kDeepItemsPerSm) * sm_count(); }
+
+int64_t sliced_split(const int32_t* hist, int64_t n_pc, int64_t n_slices, int64_t slots) {
+  if (sliced_deep(n_pc + n_slices)) return 0;
+  const int64_t warps = static_cast<int64_t>(sliced_grid(n_pc + n_slices, true)) * (kSliceThreads / 32);
+  const int64_t line = std::max<int64_t>(kSplitMinSlots, slots * 3 / (5 * warps));
+  int64_t rows = 0, split_slots = 0;
+  for (int64_t len = kSliceMaxLen; len > line; --len) {
+    const int64_t first = (rows + 31) / 32;
+    rows += hist[len];
+    split_slots += len * ((rows + 31) / 32 - first);
+  }
+  return 8 * split_slots <= slots ? (rows + 31) / 32 : 0;
+}
+
 int sliced_grid(int64_t warp_items, bool plain) {
-  const void* fn = plain ? reinterpret_cast<const void*>(spmv_sliced_kernel<EPI_COPY, false>)
-                         : reinterpret_cast<const void*>(spmv_sliced_kernel<EPI_RESID, false>);
+  const void* fn = plain ? reinterpret_cast<const void*>(spmv_sliced_kernel<EPI_COPY, SL_PLAIN>)
+                         : reinterpret_cast<const void*>(spmv_sliced_kernel<EPI_RESID, SL_PLAIN>);
   int g = occupancy_grid(fn, kSliceThreads, 0);
   int64_t need = (warp_items + kSliceThreads / 32 - 1) / (kSliceThreads / 32);
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(g, need)));
@@ -885,15 +952,16 @@ int spmv_launch(const Matrix& A, const double* x, const Epi& e, cudaStream_t s) 
   switch (A.format) {
     case GK_CSR: {
       SliceArgs b{A.rowptr, A.col, A.val, A.sl_perm, A.sl_off, A.sl_col, A.sl_val, static_cast<int>(A.n_sell),
-                  static_cast<int>(A.n_slices), A.pc, static_cast<int>(A.n_pc), A.lr_row, A.lr_off,
+                  static_cast<int>(A.n_slices), static_cast<int>(A.n_split), A.pc, static_cast<int>(A.n_pc), A.lr_row, A.lr_off,
                   static_cast<int>(A.n_lr), A.pc_sum, x};
       const bool plain = e.mode == EPI_COPY || e.mode == EPI_PLAIN;
       const int g = plain ? A.grid_sl_plain : A.grid_sl;
-      const bool deep = A.n_pc + A.n_slices <= static_cast<int64_t>(kDeepItemsPerSm) * sm_count();
+      const bool deep = sliced_deep(A.n_pc + A.n_slices);
 #define GK_SLICED(MODE)                                                                              \
   case MODE:                                                                                       \
-    if (deep) launch_pdl(spmv_sliced_kernel<MODE, true>, g, kSliceThreads, 0, s, b, e);             \
-    else launch_pdl(spmv_sliced_kernel<MODE, false>, g, kSliceThreads, 0, s, b, e);                 \
+    if (deep) launch_pdl(spmv_sliced_kernel<MODE, SL_DEEP>, g, kSliceThreads, 0, s, b, e);          \
+    else if (A.n_split > 0) launch_pdl(spmv_sliced_kernel<MODE, SL_SPLIT>, g, kSliceThreads, 0, s, b, e); \
+    else launch_pdl(spmv_sliced_kernel<MODE, SL_PLAIN>, g, kSliceThreads, 0, s, b, e);              \
     break
       switch (e.mode) {
         GK_SLICED(EPI_COPY);
