@@ -36,14 +36,14 @@
 // 17,900 cycles: direction 1,060, SpMV 2,400, update 1,440 (these three are
 // near the FP64 pipe's time for them), and per reduction 1,200 for the CTA's
 // sum, 2,300 - 3,700 until the last CTA's word is there, 990 for the sum of
-// the words, 980 for a division (260 where none is left).  A dependent FP64 add takes 68 cycles, a
-// butterfly step 145, and a warp instruction holds its quarter of the SM's
-// FP64 pipe for about 64 cycles whatever its lanes do: hence one warp per
-// value in a reduction (a quarter each) and scalars derived by one thread
-// per CTA.  CG, Jacobi, 256 x 256: 14.7 -> 8.5 ms to 1e-12 (15.6 -> 9.1 us
-// per iteration; before: an arrival counter and a release word per barrier,
-// vectors re-read from L2); BiCGSTAB, 201 x 199: 10.1 -> 4.2 ms (graph form
-// before).
+// the words, 980 for a division (260 where none is left).  A dependent FP64
+// add takes 68 cycles, a butterfly step 145, and a warp instruction holds its
+// quarter of the SM's FP64 pipe for about 64 cycles whatever its lanes do:
+// hence one warp per value in a reduction (a quarter each) and scalars
+// derived by one thread per CTA.  CG, Jacobi, 256 x 256: 14.7 -> 8.4 ms to
+// 1e-12 (15.6 -> 8.9 us per iteration; before: an arrival counter and a
+// release word per barrier, vectors re-read from L2); BiCGSTAB, 201 x 199:
+// 10.2 -> 4.0 ms (graph form before).
 //
 // Small systems (the cluster sizes of cluster_cg.cu, whose kernels keep the
 // matrices whose halo does not fit): the same kernels on 16 CTAs, the

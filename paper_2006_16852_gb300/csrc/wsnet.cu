@@ -730,21 +730,22 @@ __global__ void scale_kernel(double* __restrict__ x0, const double* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// BF16 inference on the tensor cores.  Activations are NHWC BF16 between the
-// layers (a pixel's 32 channels are 64 contiguous bytes).  The 32 -> 32
+// BF16 inference on the tensor cores.  Activations between the layers are
+// BF16 in four planes of 8 channels per image row (tc_act).  The 32 -> 32
 // layers run as an implicit GEMM on tcgen05: a tile is 128 consecutive
 // pixels of one image row (M = 128), N = 32 output channels, K = 9 taps x 32
 // input channels, issued as 18 MMAs of K = 16 (BF16 operands, FP32
-// accumulator in tensor memory).  For each kernel row ky the block stages
-// the input row y + d (ky - 1) from x0 - d to x0 + 127 + d once (zeros
-// outside the image); the three taps kx of that row are the same staged
-// window read from slot kx d on, so the MMA's A operand is the window with a
-// start address shifted by kx d rows.  Operands are K-major without
-// swizzling: a core matrix is 8 rows x 16 bytes (8 channels); rows of a
-// matrix are 16 bytes apart and its 8-channel chunks LBO bytes apart.  The
+// accumulator in tensor memory).  A block works down a strip of rows with a
+// ring of staged input rows, each from x0 - d to x0 + 127 + d (zeros outside
+// the image): bulk copies fill it, and the three taps kx of a row are the
+// same staged window read from slot kx d on, so the MMA's A operand is the
+// window with a start address shifted by kx d rows.  Operands are K-major
+// without swizzling: a core matrix is 8 rows x 16 bytes (8 channels); rows of
+// a matrix are 16 bytes apart and its 8-channel chunks LBO bytes apart.  The
 // first layer (2 input channels, K = 18 padded to 32) runs on the tensor
-// cores too (conv_first_tc_kernel); the last (1 output channel) has no GEMM
-// worth the name and runs on the CUDA cores, reading NHWC.
+// cores too, from the FP32 input (conv_first_tc_kernel); the last (1 output
+// channel) is folded into the layer before it as nine FP32 planes of
+// per-tap products, which conv_last_sum_kernel adds up.
 // ---------------------------------------------------------------------------
 
 constexpr int kTcThreads = 192;                 // 4 epilogue warps (one TMEM lane quarter each), an MMA warp, a copy warp
