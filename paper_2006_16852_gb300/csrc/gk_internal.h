@@ -227,6 +227,7 @@ struct Matrix {
   int32_t* sl_col = nullptr;
   double* sl_val = nullptr;
   int64_t n_sell = 0, n_slices = 0, sl_entries = 0;
+  bool sl_deep = false;         // 16 slots loaded ahead (sliced_deep)
   int64_t n_split = 0;          // the longest slices, taken by four warps each (sliced_split)
   // rows longer than kSliceMaxLen (n_long of them), cut into pieces of at
   // most kPieceLen consecutive entries, longest first: {row, first entry,
@@ -289,6 +290,8 @@ int spmv_max_grid(const Matrix& A);
 int merge_grid(int64_t n_tiles);
 int coo_grid(int64_t n_chunks);
 int sliced_grid(int64_t warp_items, bool plain);
+// Whether 16 slots are loaded ahead: items warps of work, longest the longest row.
+bool sliced_deep(int64_t items, int64_t longest);
 // Slices to be taken by four warps each: hist[len] rows of len entries (up to
 // kSliceMaxLen), n_pc pieces of longer rows, slots of work (32 lanes each) in all.
 int64_t sliced_split(const int32_t* hist, int64_t n_pc, int64_t n_slices, int64_t slots);

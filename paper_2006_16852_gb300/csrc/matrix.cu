@@ -715,6 +715,7 @@ extern "C" int gk_matrix_create_csr(int64_t n_rows, int64_t n_cols, int64_t nnz,
     GK_TRY(upload(&A->lr_row, lr_row, bytes, s));
     GK_TRY(upload(&A->lr_off, lr_off, bytes, s));
     GK_TRY(dalloc_async_n(&A->pc_sum, static_cast<size_t>(std::max<int32_t>(n_slot, 1)), bytes, s));
+    A->sl_deep = sliced_deep(A->n_pc + n_slices, info.maxlen);
     A->n_split = sliced_split(info.hist, A->n_pc, n_slices, static_cast<int64_t>(info.long_slots) / 32 + total / 32);
     A->grid_sl = sliced_grid(A->n_pc + A->n_slices + 3 * A->n_split, false);
     A->grid_sl_plain = sliced_grid(A->n_pc + A->n_slices + 3 * A->n_split, true);

@@ -182,6 +182,11 @@ struct SliceMinBlocks {
 // Three stages of 8 slots measured slower (25.7 and 30.5).
 constexpr int kDeepSlots = 16;
 constexpr int kDeepItemsPerSm = 16;
+// ... and with rows longer than one batch of the plain kernel: 5- and 7-point
+// matrices gain nothing from loads ahead and pay for their predicates (CG with
+// block Jacobi on 37,440 rows, 7-point: 3,074 us without, 3,099 to 3,124 with;
+// on 27,000 rows, 27-point: 2,221 and 2,011).
+constexpr int kDeepMinLen = 8;
 
 // SL_SPLIT: for matrices with a few slices much longer than a warp's share of
 // the work.  Resident warps advance at the same pace, so a warp with a slice
@@ -892,10 +897,12 @@ int merge_grid(int64_t n_tiles) {
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(g, (n_tiles + kMergeWarps - 1) / kMergeWarps)));
 }
 
-static bool sliced_deep(int64_t items) { return items <= static_cast<int64_t>(kDeepItemsPerSm) * sm_count(); }
+static bool sliced_few(int64_t items) { return items <= static_cast<int64_t>(kDeepItemsPerSm) * sm_count(); }
+
+bool sliced_deep(int64_t items, int64_t longest) { return sliced_few(items) && longest > kDeepMinLen; }
 
 int64_t sliced_split(const int32_t* hist, int64_t n_pc, int64_t n_slices, int64_t slots) {
-  if (sliced_deep(n_pc + n_slices)) return 0;
+  if (sliced_few(n_pc + n_slices)) return 0;
   const int64_t warps = static_cast<int64_t>(sliced_grid(n_pc + n_slices, true)) * (kSliceThreads / 32);
   const int64_t line = std::max<int64_t>(kSplitMinSlots, slots * 3 / (5 * warps));
   int64_t rows = 0, split_slots = 0;
@@ -956,10 +963,9 @@ int spmv_launch(const Matrix& A, const double* x, const Epi& e, cudaStream_t s) 
                   static_cast<int>(A.n_lr), A.pc_sum, x};
       const bool plain = e.mode == EPI_COPY || e.mode == EPI_PLAIN;
       const int g = plain ? A.grid_sl_plain : A.grid_sl;
-      const bool deep = sliced_deep(A.n_pc + A.n_slices);
 #define GK_SLICED(MODE)                                                                              \
   case MODE:                                                                                       \
-    if (deep) launch_pdl(spmv_sliced_kernel<MODE, SL_DEEP>, g, kSliceThreads, 0, s, b, e);          \
+    if (A.sl_deep) launch_pdl(spmv_sliced_kernel<MODE, SL_DEEP>, g, kSliceThreads, 0, s, b, e);     \
     else if (A.n_split > 0) launch_pdl(spmv_sliced_kernel<MODE, SL_SPLIT>, g, kSliceThreads, 0, s, b, e); \
     else launch_pdl(spmv_sliced_kernel<MODE, SL_PLAIN>, g, kSliceThreads, 0, s, b, e);              \
     break

@@ -23,7 +23,7 @@ def _csr(lengths, ncols, seed):
     return ptr, col.astype(np.int32), g.uniform(-1, 1, int(ptr[-1]))
 
 
-@pytest.mark.parametrize("longest", [1, 15, 16, 17, 31, 32, 33, 48, 255, 256])
+@pytest.mark.parametrize("longest", [1, 8, 9, 15, 16, 17, 31, 32, 33, 48, 255, 256])
 @pytest.mark.parametrize("n", [300, 1023])
 def test_rows_around_the_batch(gk, orc, longest, n):
     lengths = np.random.default_rng(longest).integers(0, longest + 1, n)
