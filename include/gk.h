@@ -21,7 +21,9 @@
  *    are lent for the duration of the call; gk_matrix_create_csr copies the
  *    caller's CSR arrays into library-owned storage; solvers and
  *    preconditioners share ownership of the matrix (and preconditioner) they
- *    were generated from, so the caller may destroy its handles in any order.
+ *    were generated from, so the caller may destroy its handles in any order,
+ *    also while work that uses them is still running: the call that gives up
+ *    the last reference waits for the device before it frees anything.
  *  - stream is a cudaStream_t (NULL = the legacy default stream).  All device
  *    work is enqueued on it.  gk_apply/gk_apply_adv/gk_precond_apply with
  *    device vectors are asynchronous; gk_solve returns after the solve has
@@ -200,7 +202,10 @@ GK_API int32_t gk_version(void);
  * in the requested format.  Columns must be sorted and unique within each
  * row and in [0, n_cols); rowptr[0] = 0, nondecreasing, rowptr[n_rows] = nnz.
  * Violations return GK_ERR_CSR.  GK_ELL is refused (GK_ERR_FORMAT) when its
- * padded size exceeds 8 * nnz + n_rows slots.  On success *out owns the copy. */
+ * padded size exceeds 8 * nnz + n_rows slots.  On success *out owns the copy.
+ * Its arrays are allocated on `stream` from the device's default stream-ordered
+ * memory pool (the library lets the pool keep up to 8 GB of freed memory for
+ * reuse); the call returns after the copy is complete. */
 GK_API int gk_matrix_create_csr(int64_t n_rows, int64_t n_cols, int64_t nnz, const int32_t* rowptr,
                          const int32_t* col, const void* val, int32_t dtype, int32_t format,
                          void* stream, gk_matrix* out);
@@ -231,10 +236,9 @@ GK_API int gk_apply_dot(gk_matrix A, const double* b, double* x, const double* u
  * diagonal block inverted by Gauss-Jordan elimination with partial pivoting
  * (Section 7.5).  A zero/missing diagonal or a singular block returns
  * GK_ERR_SINGULAR.  The inverse diagonal or blocks are allocated on `stream`
- * from the device's default stream-ordered memory pool (the library lets the
- * pool keep up to 8 GB of freed memory for reuse, so repeated generations do
- * not map memory again); the call returns after the generation has
- * finished (it reads back the error check). */
+ * from the device's default stream-ordered memory pool, as an operator's
+ * arrays are; the call returns after the generation has finished (it reads
+ * back the error check). */
 GK_API int gk_precond_generate(gk_matrix A, int32_t block_size, void* stream, gk_precond* out);
 
 /* z = M^{-1} r (the preconditioner as a LinOp). */

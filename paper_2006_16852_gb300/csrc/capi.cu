@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "gk_device.cuh"
 #include "gk_internal.h"
@@ -50,7 +51,47 @@ void dfree(void* p) {
 namespace {
 std::mutex g_pool_mu;
 bool g_pool_ready[64] = {};
+std::mutex g_late_mu;
+std::vector<void*> g_late[64];  // arrays whose wait in dfree_idle failed
+// A word of cudaMalloc that lives on and keeps its 2 MB chunk mapped: the wait
+// in dfree_idle, and a small solver's arrays, would otherwise map and unmap
+// one each time (97 us against 3).
+void* g_keep[64] = {};
+
+// Waits until the current device has finished all work launched so far, with
+// the free of a word of cudaMalloc, which waits for it.  (So would
+// cudaDeviceSynchronize, but that fails, and breaks the capture, while any
+// stream of any thread is being captured, where a free is allowed unless the
+// capture is in the global mode or the calling thread's own.)
+bool wait_idle() {
+  void* w = nullptr;
+  cudaError_t e = cudaMalloc(&w, 16);
+  if (e == cudaSuccess) e = cudaFree(w);
+  else if (e == cudaErrorMemoryAllocation) e = cudaDeviceSynchronize();
+  cudaGetLastError();
+  return e == cudaSuccess;
+}
 }  // namespace
+
+void dfree_idle(void* const* ptrs, size_t n) {
+  const int dev = current_device() & 63;
+  // arrays of earlier calls are freed too, if they were given up before this wait
+  std::vector<void*> all;
+  {
+    std::lock_guard<std::mutex> lock(g_late_mu);
+    all.swap(g_late[dev]);
+    if (!g_keep[dev]) cudaMalloc(&g_keep[dev], 16);
+  }
+  for (size_t i = 0; i < n; ++i)
+    if (ptrs[i]) all.push_back(ptrs[i]);
+  if (all.empty()) return;
+  if (wait_idle()) {
+    for (void* p : all) cudaFree(p);
+    return;
+  }
+  std::lock_guard<std::mutex> lock(g_late_mu);
+  g_late[dev].insert(g_late[dev].end(), all.begin(), all.end());
+}
 
 int dalloc_async(void** p, size_t bytes, int64_t* counter, cudaStream_t s) {
   *p = nullptr;

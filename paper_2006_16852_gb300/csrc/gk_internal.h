@@ -41,12 +41,17 @@ int dalloc_n(T** p, size_t n, int64_t* counter) {
 }
 void dfree(void* p);
 // Stream-ordered allocation on s from the device's default memory pool (which
-// keeps up to 8 GB of freed memory for reuse); dfree releases it.
+// keeps up to 8 GB of freed memory for reuse).  To be released by dfree_idle:
+// unlike that of dalloc's memory, the free of the pool's waits for nothing.
 int dalloc_async(void** p, size_t bytes, int64_t* counter, cudaStream_t s);
 template <class T>
 int dalloc_async_n(T** p, size_t n, int64_t* counter, cudaStream_t s) {
   return dalloc_async(reinterpret_cast<void**>(p), n * sizeof(T), counter, s);
 }
+
+// Frees arrays of the current device (of either kind, null ones skipped) once
+// the work launched on it so far has finished.
+void dfree_idle(void* const* ptrs, size_t n);
 
 // Number of SMs of the current device (cached per device).
 int sm_count();

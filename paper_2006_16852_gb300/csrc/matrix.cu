@@ -571,7 +571,9 @@ void matrix_release(Matrix* A) {
                   A->tail_rows, A->tail_rowptr, A->tail_row, A->tail_col, A->tail_val, A->tail_slot,
                   A->tail_sum, A->coo_first, A->coo_last, A->coo_head, A->coo_tail, A->partials, A->counter,
                   A->err, A->dot_st, A->stage_in, A->stage_out};
-  for (void* p : ptrs) dfree(p);
+  // applies are asynchronous, and a failed creation leaves kernels behind:
+  // the pool must not hand these arrays out before they have finished
+  dfree_idle(ptrs, sizeof(ptrs) / sizeof(ptrs[0]));
   if (prev >= 0) cudaSetDevice(prev);
   delete A;
 }

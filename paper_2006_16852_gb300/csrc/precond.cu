@@ -431,10 +431,8 @@ void precond_release(Precond* P) {
   int prev = -1;
   cudaGetDevice(&prev);
   cudaSetDevice(P->device);
-  dfree(P->dinv);
-  dfree(P->blocks);
-  dfree(P->stage_in);
-  dfree(P->stage_out);
+  void* ptrs[] = {P->dinv, P->blocks, P->stage_in, P->stage_out};
+  dfree_idle(ptrs, 4);
   matrix_release(P->A);
   if (prev >= 0) cudaSetDevice(prev);
   delete P;
