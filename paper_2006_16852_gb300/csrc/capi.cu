@@ -2,8 +2,10 @@
 // arguments, the apply calls (Section 4.2) and the reproducible dot product.
 #include <cstdarg>
 #include <cstdio>
+#include <map>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "gk_device.cuh"
@@ -131,9 +133,16 @@ int current_device() {
 }
 
 int set_smem(const void* fn, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> limits;
+  const std::pair<int, const void*> key(current_device(), fn);
+  std::lock_guard<std::mutex> lock(mu);
+  const auto at = limits.find(key);
+  if (at != limits.end() && at->second >= smem) return GK_OK;
   GK_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
   GK_TRY_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
                                    static_cast<int>(cudaSharedmemCarveoutMaxShared)));
+  limits[key] = smem;
   return GK_OK;
 }
 

@@ -60,7 +60,9 @@ int current_device();
 // Lets kernel `fn` use `smem` bytes of dynamic shared memory and asks for
 // the largest shared-memory carveout, so that as many of its blocks fit an
 // SM as its shared memory allows (with the default carveout the occupancy
-// query and the launch may settle for fewer).
+// query and the launch may settle for fewer).  The limit is the kernel's, in
+// the whole process, and only ever raised: a handle that needs less leaves it
+// where an earlier one's launches need it.
 int set_smem(const void* fn, size_t smem);
 template <typename F>
 int set_smem(F* fn, size_t smem) {

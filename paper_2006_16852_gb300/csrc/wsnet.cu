@@ -1619,7 +1619,6 @@ extern "C" int gk_wsnet_create(int32_t H, int32_t W, int32_t batch_max, const in
   GK_TRY(dalloc_n(&N->wtc, static_cast<size_t>(kTcMidLayers) * kTcPacked, by));
   GK_TRY(dalloc_n(&N->err, 1, by));
   GK_TRY_CUDA(cudaMemset(N->err, 0, sizeof(int)));
-  // (process-wide attributes: the most any network's dilations need)
   GK_TRY(set_smem(wgrad32_kernel, std::max(w32_smem(kTcMaxDil), w32_smem(32))));
   GK_TRY(set_smem(conv32_kernel<CONV_RELU>, kC32Smem));
   GK_TRY(set_smem(conv32_kernel<CONV_MASK>, kC32Smem));
