@@ -369,7 +369,13 @@ struct GridRows {
 // a square root there is about 650 cycles that every thread waits for, so
 // beta's divisor is inverted along with an earlier quotient, in another lane
 // (scale), and a norm's square root is taken only where the criteria may
-// hold: rr > tol2 implies ||r|| > tol.
+// hold: rr > tol2 implies ||r|| > tol.  An inverse that is no normal number
+// (the divisor below 5.6e-309 or above 4.5e307, as with a right-hand side
+// scaled near 1e-150 or 1e150) is not used: beta is then the quotient itself.
+__device__ __forceinline__ bool gr_normal(double v) {
+  return ((static_cast<unsigned int>(__double2hiint(v)) >> 20) & 0x7ffu) - 1u < 0x7feu;
+}
+
 struct GrScalars {
   double rho, rho_prev, alpha, omega, beta, scale, rr, ss, rnorm0, bnorm, ref, tol, tol2;
   long long iter, spmvs;
@@ -562,7 +568,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
               [&](int warp, int lane, const double* tt) {
                 if (lane != 0) return;
                 if (warp == 0) {
-                  sc.beta = tt[0] * sc.scale;
+                  sc.beta = gr_normal(sc.scale) ? tt[0] * sc.scale : tt[0] / sc.rho;
                   sc.rho = tt[0];
                 } else {
                   sc.iter += 1;
@@ -632,7 +638,8 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
     if (!isfinite(rho)) sc.stop = GK_STOP_NAN;
     else if (rho == 0.0) sc.stop = GK_STOP_BREAKDOWN;
     else {
-      sc.beta = rho * sc.scale;  // scale = (alpha / omega) / the previous rho
+      // scale = (alpha / omega) / the previous rho
+      sc.beta = gr_normal(sc.scale) ? rho * sc.scale : (rho / sc.rho) * (sc.alpha / sc.omega);
       sc.rho = rho;
     }
   };
@@ -696,7 +703,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
                   const double rhv = tt[0];
                   const double q = (lane == 0 ? sc.rho : 1.0) / rhv;
                   if (lane == 1) {
-                    sc.scale = q;
+                    sc.scale = gr_normal(q) ? q : nan("");
                     return;
                   }
                   sc.spmvs += 1;
@@ -736,7 +743,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
                 // (alpha / omega) / rho = (1 / r^.v) (t.t / s.t)
                 const double q = tt[lane == 0 ? 0 : 2] / tt[lane == 0 ? 2 : 0];
                 if (lane == 1) {
-                  sc.scale *= q;
+                  sc.scale = gr_normal(q) ? sc.scale * q : nan("");
                   return;
                 }
                 if (!isfinite(tt[2]) || !isfinite(tt[0])) sc.om_stop = GK_STOP_NAN;
