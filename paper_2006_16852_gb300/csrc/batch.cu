@@ -49,11 +49,15 @@ struct BatchClass {
 
 // The vectors of the solve at hand, in device memory: the graph of a
 // configuration reads them from here, so that other vectors need no other
-// graph (building one takes about a millisecond).
+// graph (building one takes about a millisecond).  batch_io_kernel stores
+// them, by value: a copy from the host's memory would have to find it
+// unchanged when the stream gets there, after the call has returned.
 struct BatchIo {
   const double* b;
   double* x;
 };
+
+__global__ void batch_io_kernel(BatchIo* io, const double* b, double* x) { *io = {b, x}; }
 
 struct BatchArgs {
   const int32_t* sys_ptr;
@@ -1269,8 +1273,8 @@ extern "C" int gk_batch_solve(gk_batch h, int32_t kind, int32_t jacobi, const gk
       }
       memcpy(B->key, key, sizeof(key));
     }
-    const BatchIo io = {static_cast<const double*>(b), static_cast<double*>(x)};
-    cudaError_t e = cudaMemcpyAsync(B->io, &io, sizeof(io), cudaMemcpyHostToDevice, s);
+    batch_io_kernel<<<1, 1, 0, s>>>(B->io, static_cast<const double*>(b), static_cast<double*>(x));
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaGraphLaunch(B->exec, s);
     if (e != cudaSuccess) {
       rc = cuda_error(e, "gk_batch_solve: graph launch");
@@ -1325,8 +1329,8 @@ extern "C" int gk_batch_autotune(gk_batch h, int32_t kind, int32_t jacobi, const
   int chosen[kBatchClasses] = {};
   do {
     if (!B->xtune && (rc = dalloc_n(&B->xtune, static_cast<size_t>(B->n_rows), &B->device_bytes))) break;
-    const BatchIo io = {static_cast<const double*>(b), B->xtune};
-    cudaError_t e = cudaMemcpyAsync(B->io, &io, sizeof(io), cudaMemcpyHostToDevice, s);
+    batch_io_kernel<<<1, 1, 0, s>>>(B->io, static_cast<const double*>(b), B->xtune);
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e != cudaSuccess) {
