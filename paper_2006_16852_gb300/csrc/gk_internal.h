@@ -381,7 +381,7 @@ struct Solver {
   size_t cl_smem = 0;       // ... dynamic shared memory per CTA
   int gr_grid = 0;          // GK_CG, GK_BICGSTAB mid-size form: CTAs of the cooperative launch (0: not available)
   int gr_rpt = 1, gr_rows = 0;
-  bool gr_stage = false;            // its CTAs' rows of the matrix staged in shared memory
+  int gr_src = 0;                   // where its CTAs read their rows of the matrix (grid_cg.cu)
   int gr_nnz = 0;
   size_t gr_smem = 0;
   int gr_halo_cap = 0;              // its largest halo

@@ -305,9 +305,14 @@ __device__ __forceinline__ bool grid_total(const GridArgs& a, GridRed& red, unsi
 }
 
 // The CTA's rows of the matrix (row pointers relative to the CTA's first
-// entry, codes, values), in shared memory if they fit, and its halo.
-template <bool STAGE>
+// entry, codes, values), in shared memory if they fit (SRC_STAGED), and its
+// halo.
+enum GridSrc { SRC_STAGED = 0, SRC_SHORT = 1, SRC_LONG = 2 };
+constexpr int kGrLongRow = 16;  // SRC_LONG: some row has more entries
+
+template <int SRC>
 struct GridRows {
+  static constexpr bool STAGE = SRC == SRC_STAGED;
   const int32_t* rp;
   const int32_t* code;
   const double* val;
@@ -342,11 +347,53 @@ struct GridRows {
 
   // sum_k val_k loc[code_k] of the local row l in increasing k (the oracle's
   // ordered SpMV); entries in groups of 8 so that their loads are in flight
-  // together.
+  // together.  Rows read from memory are bound by the L1 lookups, one per
+  // thread and load, since a warp's rows lie far apart: from the first entry
+  // on a 16-byte boundary of the codes on, long rows are read 16 bytes at a
+  // time, 6 loads for 8 entries instead of 16.  Us per iteration, one entry a
+  // load / this form / the kernels of cluster_cg.cu: CG on 61 diagonals,
+  // 16,000 rows 76.8 / 42.6 / 66.5, 81 diagonals, 4,000 rows 40.0 / 19.7 /
+  // 32.8, 27-point 32^3 59.8 / 36.4 / 53.1; BiCGSTAB on the first two 142 / 81 / 111
+  // and 77.7 / 37.4 / 57.3.  Rows of up to kGrLongRow entries are two groups
+  // at most, and the steps to and from the boundary cost them more (9
+  // diagonals 19.4 against 21.5); matrices of such rows alone have kernels
+  // without the other form, whose code costs theirs 1 to 4 %.
   __device__ __forceinline__ double apply(int l, const double* loc) const {
     double s = 0.0;
     int k = STAGE ? rp[l] : __ldg(rp + l);
     const int k1 = STAGE ? rp[l + 1] : __ldg(rp + l + 1);
+    if (SRC == SRC_LONG && k1 - k > kGrLongRow) {
+      const int ka = (k + 3) & ~3;
+      int cp[3];
+      double vp[3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        cp[u] = 0;
+        vp[u] = 0.0;
+        if (k + u < ka) {
+          cp[u] = __ldg(code + k + u);
+          vp[u] = __ldg(val + k + u);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (k + u < ka) s = fma(vp[u], loc[cp[u]], s);
+      for (k = ka; k + 8 <= k1; k += 8) {
+        int4 c[2];
+        double2 v[4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) c[u] = __ldg(reinterpret_cast<const int4*>(code + k) + u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(reinterpret_cast<const double2*>(val + k) + u);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          s = fma(v[2 * u].x, loc[c[u].x], s);
+          s = fma(v[2 * u].y, loc[c[u].y], s);
+          s = fma(v[2 * u + 1].x, loc[c[u].z], s);
+          s = fma(v[2 * u + 1].y, loc[c[u].w], s);
+        }
+      }
+    }
     for (; k < k1; k += 8) {
       double v[8], w[8];
 #pragma unroll
@@ -458,7 +505,7 @@ __device__ __forceinline__ void gr_store_state(SolverState* st, const GrScalars&
 //                                       the halo's z fetched meanwhile
 //   criteria; beta = rho' / rho
 // Shared memory: p of own rows and halo, z of the halo, the staged rows.
-template <int PK, int RPT, bool STAGE, bool CLUSTER>
+template <int PK, int RPT, int SRC, bool CLUSTER>
 __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
   extern __shared__ double loc[];
   __shared__ GridRed red;
@@ -467,7 +514,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
   const int R = a.rows_per_cta;
   double* const ph = loc + R;            // p of the halo
   double* const zh = ph + a.halo_cap;    // z of the halo
-  GridRows<STAGE> A;
+  GridRows<SRC> A;
   A.init(a, zh + a.halo_cap);
   const int row0 = A.row0, H = A.H;
   SolverState* st = a.st;
@@ -600,7 +647,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
 // reduction in every iteration and costs one SpMV in the last.)
 // Shared memory: the SpMV's input on own rows and halo; p^, z and v^ of the
 // halo; the staged rows.
-template <int PK, int RPT, bool STAGE, bool CLUSTER>
+template <int PK, int RPT, int SRC, bool CLUSTER>
 __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
   extern __shared__ double loc[];
   __shared__ GridRed red;
@@ -611,7 +658,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
   double* const ph_h = in_h + a.halo_cap;
   double* const z_h = ph_h + a.halo_cap;
   double* const vh_h = z_h + a.halo_cap;
-  GridRows<STAGE> A;
+  GridRows<SRC> A;
   A.init(a, vh_h + a.halo_cap);
   const int row0 = A.row0, H = A.H;
   SolverState* st = a.st;
@@ -877,32 +924,40 @@ __global__ void __launch_bounds__(kGrPlanThreads) gr_halo_kernel(const int32_t* 
 
 using GrKernel = void (*)(GridArgs);
 
-template <int PK, bool STAGE, bool CLUSTER>
+template <int PK, int SRC, bool CLUSTER>
 GrKernel pick_rpt(int kind, int rpt) {
   if (kind == GK_BICGSTAB) {
     switch (rpt) {
-      case 1: return bicg_grid_kernel<PK, 1, STAGE, CLUSTER>;
-      case 2: return bicg_grid_kernel<PK, 2, STAGE, CLUSTER>;
-      default: return bicg_grid_kernel<PK, 4, STAGE, CLUSTER>;
+      case 1: return bicg_grid_kernel<PK, 1, SRC, CLUSTER>;
+      case 2: return bicg_grid_kernel<PK, 2, SRC, CLUSTER>;
+      default: return bicg_grid_kernel<PK, 4, SRC, CLUSTER>;
     }
   }
   switch (rpt) {
-    case 1: return cg_grid_kernel<PK, 1, STAGE, CLUSTER>;
-    case 2: return cg_grid_kernel<PK, 2, STAGE, CLUSTER>;
-    case 4: return cg_grid_kernel<PK, 4, STAGE, CLUSTER>;
-    default: return cg_grid_kernel<PK, 8, STAGE, CLUSTER>;
+    case 1: return cg_grid_kernel<PK, 1, SRC, CLUSTER>;
+    case 2: return cg_grid_kernel<PK, 2, SRC, CLUSTER>;
+    case 4: return cg_grid_kernel<PK, 4, SRC, CLUSTER>;
+    default: return cg_grid_kernel<PK, 8, SRC, CLUSTER>;
   }
 }
 
-template <bool CLUSTER>
-GrKernel pick_pk(int kind, int pk, int rpt, bool stage) {
-  if (pk == PREC_SCALAR)
-    return stage ? pick_rpt<PREC_SCALAR, true, CLUSTER>(kind, rpt) : pick_rpt<PREC_SCALAR, false, CLUSTER>(kind, rpt);
-  return stage ? pick_rpt<PREC_NONE, true, CLUSTER>(kind, rpt) : pick_rpt<PREC_NONE, false, CLUSTER>(kind, rpt);
+template <int PK, bool CLUSTER>
+GrKernel pick_src(int kind, int rpt, int src) {
+  if (src == SRC_STAGED) return pick_rpt<PK, SRC_STAGED, CLUSTER>(kind, rpt);
+  // fewer rows a thread, or BiCGSTAB's half as many, are staged unless they are long
+  if (src == SRC_SHORT && kind == GK_CG && rpt == 4) return cg_grid_kernel<PK, 4, SRC_SHORT, CLUSTER>;
+  if (src == SRC_SHORT && kind == GK_CG && rpt == 8) return cg_grid_kernel<PK, 8, SRC_SHORT, CLUSTER>;
+  return pick_rpt<PK, SRC_LONG, CLUSTER>(kind, rpt);
 }
 
-GrKernel pick(const Solver& S, int rpt, bool stage, bool cluster) {
-  return cluster ? pick_pk<true>(S.kind, S.pk, rpt, stage) : pick_pk<false>(S.kind, S.pk, rpt, stage);
+template <bool CLUSTER>
+GrKernel pick_pk(int kind, int pk, int rpt, int src) {
+  return pk == PREC_SCALAR ? pick_src<PREC_SCALAR, CLUSTER>(kind, rpt, src)
+                           : pick_src<PREC_NONE, CLUSTER>(kind, rpt, src);
+}
+
+GrKernel pick(const Solver& S, int rpt, int src, bool cluster) {
+  return cluster ? pick_pk<true>(S.kind, S.pk, rpt, src) : pick_pk<false>(S.kind, S.pk, rpt, src);
 }
 
 cudaLaunchConfig_t cluster_config(size_t smem, cudaStream_t s, cudaLaunchAttribute* attr) {
@@ -976,7 +1031,8 @@ int grid_cg_plan(Solver* S, bool cluster) {
   const size_t staged = 12 * static_cast<size_t>(most) + 4 * static_cast<size_t>(R + 1);
   const bool stage = vectors + staged <= kGrSmemMax;
   const size_t smem = vectors + (stage ? staged : 0);
-  GrKernel k = pick(*S, rpt, stage, cluster);
+  const int src = stage ? SRC_STAGED : longest > kGrLongRow ? SRC_LONG : SRC_SHORT;
+  GrKernel k = pick(*S, rpt, src, cluster);
   bool fits = set_smem(k, smem) == GK_OK;
   if (fits && cluster) {
     cudaLaunchAttribute attr[1];
@@ -1005,7 +1061,7 @@ int grid_cg_plan(Solver* S, bool cluster) {
   S->gr_rpt = rpt;
   S->gr_rows = static_cast<int>(R);
   S->gr_halo_cap = static_cast<int>(cap);
-  S->gr_stage = stage;
+  S->gr_src = src;
   S->gr_nnz = stage ? static_cast<int>(most) : 0;
   S->gr_smem = smem;
   S->gr_epoch = 1;
@@ -1046,7 +1102,7 @@ int grid_cg_solve(Solver* S, bool cluster, cudaStream_t s) {
   a.rows_per_cta = S->gr_rows;
   a.stage_nnz = S->gr_nnz;
   GK_TRY_CUDA(cudaMemsetAsync(a.abort_, 0, sizeof(unsigned int), s));
-  GrKernel k = pick(*S, S->gr_rpt, S->gr_stage, cluster);
+  GrKernel k = pick(*S, S->gr_rpt, S->gr_src, cluster);
   if (cluster) {
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = cluster_config(S->gr_smem, s, attr);

@@ -1,0 +1,81 @@
+"""The one-launch CG and BiCGSTAB where a CTA's rows of the matrix do not fit
+its shared memory and are read from memory, long rows 16 bytes at a time from
+the first aligned entry on: rows of 1 to 70 entries that start at every
+offset, in the cluster and in the grid form."""
+import time
+
+import numpy as np
+import pytest
+
+import workloads as W
+from helpers import to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+def _ragged_band(n, reach, seed):
+    """Symmetric, diagonally dominant; row i is coupled to a run of up to
+    `reach` neighbours of random length, every 7th row to none."""
+    rng = np.random.default_rng(seed)
+    i = np.arange(n)
+    lens = rng.integers(0, reach + 1, n)
+    lens[::7] = 0
+    lens = np.minimum(lens, n - 1 - i)
+    r = np.repeat(i, lens)
+    d = np.arange(r.size) - np.repeat(np.cumsum(lens) - lens, lens) + 1
+    c = r + d
+    v = -rng.uniform(0.1, 1.0, r.size)
+    diag = 1.0 + np.bincount(r, -v, n) + np.bincount(c, -v, n)
+    return W._coo_to_csr(n, np.concatenate([r, c, i]), np.concatenate([c, r, i]), np.concatenate([v, v, diag]))
+
+
+def _solver(gk, A, kind, prec, **crit):
+    M = gk.Matrix(*[to_dev(a) for a in A])
+    return gk.Solver(M, gk.Precond(M, 1) if prec else None, kind, **crit)
+
+
+@pytest.mark.parametrize("kind", ["cg", "bicgstab"])
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,reach", [(16000, 45), (16001, 33), (120000, 35), (130003, 30)])
+def test_against_graph_form(gk, orc, kind, prec, n, reach):
+    A = _ragged_band(n, reach, n)
+    share = -(-n // (16 if n < 32769 else 152))
+    assert 12 * A[1].size * share // n > 216 * 1024  # not staged
+    b = orc.spmv(A, W.uniform_vector(n, 11))
+    out = []
+    for check_every in (0, -1):
+        S = _solver(gk, A, kind, prec, max_iters=4000, reduction_factor=1e-10, check_every=check_every)
+        x = to_dev(np.zeros(n))
+        st = gk.solve(S, to_dev(b), x)
+        assert st.stop_reason == gk.STOP_CONVERGED and st.device_error == 0
+        assert np.linalg.norm(b - orc.spmv(A, to_np(x))) <= 1.5e-10 * np.linalg.norm(b)
+        out.append(st)
+    assert out[0].form == (gk.FORM_CLUSTER if n < 32769 else gk.FORM_GRID) and out[1].form == gk.FORM_GRAPH
+    slack = max(2, out[1].iters * 3 // 100) if kind == "cg" else max(3, out[1].iters // 4)
+    assert abs(out[0].iters - out[1].iters) <= slack, (out[0].iters, out[1].iters)
+
+
+def test_long_rows_are_not_slower_than_across_the_cluster(gk):
+    """61 diagonals on 16,000 rows: the kernels that read the direction vector
+    across the cluster took 66.5 us an iteration, this form with one entry per
+    load 77 us, with 16-byte loads 43."""
+    import torch
+    n, half = 16000, 30
+    i = np.arange(n)
+    r, c = [i], [i]
+    for d in range(1, half + 1):
+        r += [i[d:], i[:-d]]
+        c += [i[:-d], i[d:]]
+    r, c = np.concatenate(r), np.concatenate(c)
+    A = W._coo_to_csr(n, r, c, np.where(r == c, 2.0 * half + 1.0, -1.0))
+    S = _solver(gk, A, "cg", 1, max_iters=100, reduction_factor=1e-300)
+    b = to_dev(W.uniform_vector(n, 12))
+    best = 1.0
+    for _ in range(5):
+        x = torch.zeros_like(b)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        st = gk.solve(S, b, x)
+        best = min(best, time.perf_counter() - t0)
+    assert st.form == gk.FORM_CLUSTER and st.iters == 100
+    assert best <= 100 * 60e-6, best
