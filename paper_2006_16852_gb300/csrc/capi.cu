@@ -55,10 +55,8 @@ std::mutex g_pool_mu;
 bool g_pool_ready[64] = {};
 std::mutex g_late_mu;
 std::vector<void*> g_late[64];  // arrays whose wait in dfree_idle failed
-// A word of cudaMalloc that lives on and keeps its 2 MB chunk mapped: the wait
-// in dfree_idle, and a small solver's arrays, would otherwise map and unmap
-// one each time (97 us against 3).
-void* g_keep[64] = {};
+std::mutex g_keep_mu;
+void* g_keep[64][2] = {};
 
 // Waits until the current device has finished all work launched so far, with
 // the free of a word of cudaMalloc, which waits for it.  (So would
@@ -75,6 +73,14 @@ bool wait_idle() {
 }
 }  // namespace
 
+void keep_chunks() {
+  const int dev = current_device() & 63;
+  std::lock_guard<std::mutex> lock(g_keep_mu);
+  if (!g_keep[dev][0] && cudaMalloc(&g_keep[dev][0], 16) != cudaSuccess) g_keep[dev][0] = nullptr;
+  if (!g_keep[dev][1] && cudaMallocHost(&g_keep[dev][1], 16) != cudaSuccess) g_keep[dev][1] = nullptr;
+  cudaGetLastError();
+}
+
 void dfree_idle(void* const* ptrs, size_t n) {
   const int dev = current_device() & 63;
   // arrays of earlier calls are freed too, if they were given up before this wait
@@ -82,8 +88,8 @@ void dfree_idle(void* const* ptrs, size_t n) {
   {
     std::lock_guard<std::mutex> lock(g_late_mu);
     all.swap(g_late[dev]);
-    if (!g_keep[dev]) cudaMalloc(&g_keep[dev], 16);
   }
+  keep_chunks();
   for (size_t i = 0; i < n; ++i)
     if (ptrs[i]) all.push_back(ptrs[i]);
   if (all.empty()) return;

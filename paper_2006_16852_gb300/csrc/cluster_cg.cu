@@ -660,6 +660,12 @@ int cluster_cg_plan(Solver* S) {
   if (n < 1 || n > static_cast<int64_t>(kClCtas) * kClThreads * max_rpt) return GK_OK;
   int lg = 0;
   while ((static_cast<int64_t>(kClCtas) << lg) < n) ++lg;
+  // the halo form of the same cluster, where the halos fit shared memory
+  GK_TRY(grid_cg_plan(S, true));
+  if (S->gr_grid > 0) {
+    S->cl_lg = lg;
+    return GK_OK;
+  }
   const int rpt = std::max(1, (1 << lg) / kClThreads);
   // the most entries any CTA's rows hold: stage them if they fit
   std::vector<int32_t> rp(static_cast<size_t>(n) + 1);
@@ -693,8 +699,7 @@ int cluster_cg_plan(Solver* S) {
   S->cl_stage = stage;
   S->cl_nnz = stage ? static_cast<int>(most) : 0;
   S->cl_smem = smem;
-  // the halo form of the same cluster, where the halos fit shared memory
-  return grid_cg_plan(S, true);
+  return GK_OK;
 }
 
 int cluster_cg_solve(Solver* S, cudaStream_t s) {

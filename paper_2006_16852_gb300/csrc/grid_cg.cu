@@ -860,8 +860,10 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
 
 // The halo of every CTA: a bitmap of the columns of its rows that other CTAs
 // own (n bits of shared memory), and their ranks.  With halo_col null only
-// the counts are written; else also the halo's columns in increasing order
-// and, per entry of the matrix, the place of its column in the CTA's slice.
+// counts are written, of the halos, then of the CTAs' entries and of those of
+// their longest rows (halo_n[3][grid]); else the halos' counts, their columns
+// in increasing order and, per entry of the matrix, the place of its column
+// in the CTA's slice.
 __global__ void __launch_bounds__(kGrPlanThreads) gr_halo_kernel(const int32_t* __restrict__ rowptr,
                                                                  const int32_t* __restrict__ col, int n, int R,
                                                                  int halo_cap, int32_t* __restrict__ halo_n,
@@ -869,13 +871,20 @@ __global__ void __launch_bounds__(kGrPlanThreads) gr_halo_kernel(const int32_t* 
                                                                  int32_t* __restrict__ code) {
   extern __shared__ uint32_t bits[];  // ceil(n / 32) words, then as many ranks
   __shared__ int wsum[kGrPlanThreads / 32];
+  __shared__ int s_longest;
   const int nw = (n + 31) / 32;
   int* rank = reinterpret_cast<int*>(bits + nw);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int row0 = min(static_cast<int>(blockIdx.x) * R, n), rows = min(R, n - row0);
   const int e0 = rowptr[row0], e1 = rowptr[row0 + rows];
   for (int w = t; w < nw; w += kGrPlanThreads) bits[w] = 0u;
+  if (t == 0) s_longest = 0;
   __syncthreads();
+  if (!halo_col) {
+    int longest = 0;
+    for (int l = t; l < rows; l += kGrPlanThreads) longest = max(longest, rowptr[row0 + l + 1] - rowptr[row0 + l]);
+    atomicMax(&s_longest, longest);
+  }
   for (int k = e0 + t; k < e1; k += kGrPlanThreads) {
     const int c = col[k];
     if (c < row0 || c >= row0 + rows) atomicOr(bits + (c >> 5), 1u << (c & 31));
@@ -902,7 +911,13 @@ __global__ void __launch_bounds__(kGrPlanThreads) gr_halo_kernel(const int32_t* 
     at += __popc(bits[w]);
   }
   if (t == kGrPlanThreads - 1) halo_n[blockIdx.x] = at;
-  if (!halo_col) return;
+  if (!halo_col) {
+    if (t == 0) {
+      halo_n[gridDim.x + blockIdx.x] = e1 - e0;
+      halo_n[2 * gridDim.x + blockIdx.x] = s_longest;
+    }
+    return;
+  }
   __syncthreads();
   int32_t* out = halo_col + static_cast<int64_t>(blockIdx.x) * halo_cap;
   for (int w = t; w < nw; w += kGrPlanThreads) {
@@ -982,7 +997,8 @@ constexpr size_t kGrSmemMax = 216 * 1024;
 }  // namespace
 
 // cluster: the plan of the 16-CTA form (the caller has checked that the
-// cluster form applies); else of the cooperative grid.
+// cluster form applies); else of the cooperative grid.  Its arrays come from
+// the pool, like the operator's.
 int grid_cg_plan(Solver* S, bool cluster) {
   S->gr_grid = 0;
   if ((S->kind != GK_CG && S->kind != GK_BICGSTAB) || S->pk == PREC_BLOCK) return GK_OK;
@@ -1001,27 +1017,19 @@ int grid_cg_plan(Solver* S, bool cluster) {
   int rpt = 1;
   while (static_cast<int64_t>(rpt) * kGrThreads < R) rpt *= 2;
   if (G > kGrMaxCtas || rpt > (bi ? kGrMaxRptBi : kGrMaxRptCg)) return GK_OK;
-  // longest row (one thread per row), the most entries a CTA's rows hold
-  std::vector<int32_t> rp(static_cast<size_t>(n) + 1);
-  GK_TRY_CUDA(cudaMemcpy(rp.data(), S->A->rowptr, sizeof(int32_t) * rp.size(), cudaMemcpyDeviceToHost));
-  int32_t longest = 0;
-  for (int64_t i = 0; i < n; ++i) longest = std::max(longest, rp[i + 1] - rp[i]);
-  if (longest > kGrMaxRowLen && !cluster) return GK_OK;
-  int64_t most = 0;
-  for (int c = 0; c < G; ++c) {
-    const int64_t lo = std::min<int64_t>(c * R, n), hi = std::min<int64_t>((c + 1) * R, n);
-    most = std::max<int64_t>(most, rp[hi] - rp[lo]);
-  }
-  // halo sizes, then the lists
+  // the CTAs' halos, entries and longest rows, then the lists
   const size_t plan_smem = 8 * static_cast<size_t>((n + 31) / 32);
   GK_TRY(set_smem(gr_halo_kernel, plan_smem));
-  GK_TRY(dalloc_n(&S->gr_halo_n, static_cast<size_t>(G), &S->device_bytes));
+  GK_TRY(dalloc_async_n(&S->gr_halo_n, static_cast<size_t>(3 * G), &S->device_bytes, nullptr));
   gr_halo_kernel<<<G, kGrPlanThreads, plan_smem>>>(S->A->rowptr, S->A->col, static_cast<int>(n), static_cast<int>(R),
                                                    0, S->gr_halo_n, nullptr, nullptr);
   GK_TRY_CUDA(cudaGetLastError());
-  std::vector<int32_t> halo(static_cast<size_t>(G));
-  GK_TRY_CUDA(cudaMemcpy(halo.data(), S->gr_halo_n, sizeof(int32_t) * halo.size(), cudaMemcpyDeviceToHost));
-  const int64_t cap = std::max<int32_t>(1, *std::max_element(halo.begin(), halo.end()));
+  std::vector<int32_t> info(static_cast<size_t>(3 * G));
+  GK_TRY_CUDA(cudaMemcpy(info.data(), S->gr_halo_n, sizeof(int32_t) * info.size(), cudaMemcpyDeviceToHost));
+  const auto most_of = [&](int k) { return *std::max_element(info.begin() + k * G, info.begin() + (k + 1) * G); };
+  const int64_t cap = std::max<int32_t>(1, most_of(0)), most = most_of(1);
+  const int32_t longest = most_of(2);
+  if (longest > kGrMaxRowLen && !cluster) return GK_OK;  // one thread per row: no long rows
   const size_t vectors = sizeof(double) * static_cast<size_t>(R + (bi ? 4 : 2) * cap);
   // Scattered columns, whose halo does not fit: the graph form.  Measured with
   // halos gathered from global memory instead (us per iteration, graph form
@@ -1049,14 +1057,15 @@ int grid_cg_plan(Solver* S, bool cluster) {
     return GK_OK;
   }
   const size_t n_words = static_cast<size_t>(2) * kGrCopies * kGrMaxK * G + 1, n_vec = static_cast<size_t>(bi ? 4 : 2) * n;
-  GK_TRY(dalloc_n(&S->gr_words, n_words + n_vec, &S->device_bytes));
-  GK_TRY(dalloc_n(&S->gr_halo_col, static_cast<size_t>(G) * cap, &S->device_bytes));
-  GK_TRY(dalloc_n(&S->gr_code, static_cast<size_t>(std::max<int64_t>(S->A->nnz, 1)), &S->device_bytes));
+  GK_TRY(dalloc_async_n(&S->gr_words, n_words + n_vec, &S->device_bytes, nullptr));
+  GK_TRY(dalloc_async_n(&S->gr_halo_col, static_cast<size_t>(G) * cap, &S->device_bytes, nullptr));
+  GK_TRY(dalloc_async_n(&S->gr_code, static_cast<size_t>(std::max<int64_t>(S->A->nnz, 1)), &S->device_bytes, nullptr));
   GK_TRY_CUDA(cudaMemset(S->gr_words, 0, (n_words + n_vec) * sizeof(ulonglong2)));
   gr_halo_kernel<<<G, kGrPlanThreads, plan_smem>>>(S->A->rowptr, S->A->col, static_cast<int>(n), static_cast<int>(R),
                                                    static_cast<int>(cap), S->gr_halo_n, S->gr_halo_col, S->gr_code);
   GK_TRY_CUDA(cudaGetLastError());
-  GK_TRY_CUDA(cudaDeviceSynchronize());
+  // (the caller waits for the null stream; the device's wait, which was here,
+  // breaks other threads' captures)
   S->gr_grid = G;
   S->gr_rpt = rpt;
   S->gr_rows = static_cast<int>(R);

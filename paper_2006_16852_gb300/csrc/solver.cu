@@ -507,14 +507,12 @@ void solver_release(Solver* S) {
   if (S->exec) cudaGraphExecDestroy(S->exec);
   if (S->graph) cudaGraphDestroy(S->graph);
   if (S->cs) cudaStreamDestroy(S->cs);
-  for (double* v : {S->b, S->x, S->r, S->p, S->q, S->z, S->rh, S->ph, S->s, S->sh, S->t}) dfree(v);
+  void* const pooled[] = {S->b, S->x, S->r,  S->p, S->q,        S->z,         S->rh,         S->ph,
+                          S->s, S->sh, S->t, S->gr_words, S->gr_halo_n, S->gr_halo_col, S->gr_code};
+  dfree_idle(pooled, sizeof(pooled) / sizeof(pooled[0]));
   dfree(S->st);
   dfree(S->partials);
   dfree(S->counter);
-  dfree(S->gr_words);
-  dfree(S->gr_halo_n);
-  dfree(S->gr_halo_col);
-  dfree(S->gr_code);
   if (S->h_st) cudaFreeHost(S->h_st);
   ir_release(S->ir);
   gmres_release(S->gm);
@@ -706,8 +704,10 @@ int build_graph(Solver& S) {
   return GK_OK;
 }
 
+// From the pool, like the operator's arrays: mapped and unmapped for each
+// solver of 65,536 rows, five vectors take 150 us.
 int alloc_vec(double** v, int64_t n, int64_t* bytes) {
-  return dalloc_n(v, static_cast<size_t>(std::max<int64_t>(n, 1)), bytes);
+  return dalloc_async_n(v, static_cast<size_t>(std::max<int64_t>(n, 1)), bytes, nullptr);
 }
 
 }  // namespace
@@ -748,6 +748,7 @@ extern "C" int gk_solver_generate(gk_matrix hA, gk_precond hP, int32_t kind, con
   S->n = A->n_rows;
   int64_t* by = &S->device_bytes;
   int rc = GK_OK;
+  keep_chunks();
   do {
     if ((rc = alloc_vec(&S->b, S->n, by)) || (rc = alloc_vec(&S->x, S->n, by)) ||
         (rc = alloc_vec(&S->r, S->n, by)) || (rc = alloc_vec(&S->p, S->n, by)) ||
@@ -782,8 +783,13 @@ extern "C" int gk_solver_generate(gk_matrix hA, gk_precond hP, int32_t kind, con
     }
     if (kind == GK_IR_CG && (rc = ir_generate(S))) break;
     if (kind == GK_GMRES && (rc = gmres_generate(S))) break;
-    if ((kind == GK_CG || kind == GK_BICGSTAB) && (rc = cluster_cg_plan(S))) break;
-    if ((kind == GK_CG || kind == GK_BICGSTAB) && S->cl_lg < 0 && (rc = grid_cg_plan(S, false))) break;
+    // the one-launch forms, where gk_solve may take them
+    const bool one = (kind == GK_CG || kind == GK_BICGSTAB) && crit->check_every == 0 && !(crit->time_limit_s > 0);
+    if (one && (rc = cluster_cg_plan(S))) break;
+    if (one && S->cl_lg < 0 && (rc = grid_cg_plan(S, false))) break;
+    // the null stream's allocations and stores come before any stream's solve
+    e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess) rc = cuda_error(e, "solver set-up");
   } while (false);
   if (prev != A->device) cudaSetDevice(prev);
   if (rc != GK_OK) return rc;
