@@ -22,8 +22,10 @@
  *    caller's CSR arrays into library-owned storage; solvers and
  *    preconditioners share ownership of the matrix (and preconditioner) they
  *    were generated from, so the caller may destroy its handles in any order,
- *    also while work that uses them is still running: the call that gives up
- *    the last reference waits for the device before it frees anything.
+ *    also while work that uses them is still running: what has been used on
+ *    the legacy default stream alone is freed in that stream's order, and the
+ *    call that gives up the last reference to anything else waits for the
+ *    device.
  *  - stream is a cudaStream_t (NULL = the legacy default stream).  All device
  *    work is enqueued on it.  gk_apply/gk_apply_adv/gk_precond_apply with
  *    device vectors are asynchronous; gk_solve returns after the solve has

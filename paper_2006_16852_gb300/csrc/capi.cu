@@ -54,7 +54,7 @@ namespace {
 std::mutex g_pool_mu;
 bool g_pool_ready[64] = {};
 std::mutex g_late_mu;
-std::vector<void*> g_late[64];  // arrays whose wait in dfree_idle failed
+std::vector<void*> g_late[64];  // arrays that dfree_pooled could not free
 std::mutex g_keep_mu;
 void* g_keep[64][2] = {};
 
@@ -81,24 +81,32 @@ void keep_chunks() {
   cudaGetLastError();
 }
 
-void dfree_idle(void* const* ptrs, size_t n) {
+void dfree_pooled(void* const* ptrs, size_t n, const StreamUse& use) {
   const int dev = current_device() & 63;
-  // arrays of earlier calls are freed too, if they were given up before this wait
-  std::vector<void*> all;
-  {
+  const bool wait = use.other.load(std::memory_order_relaxed);
+  std::vector<void*> all, failed;
+  if (wait) {
+    // with the arrays of earlier calls, if they were given up before this wait
     std::lock_guard<std::mutex> lock(g_late_mu);
     all.swap(g_late[dev]);
   }
-  keep_chunks();
   for (size_t i = 0; i < n; ++i)
     if (ptrs[i]) all.push_back(ptrs[i]);
   if (all.empty()) return;
-  if (wait_idle()) {
-    for (void* p : all) cudaFree(p);
-    return;
+  if (wait) keep_chunks();
+  if (wait && !wait_idle()) {
+    failed.swap(all);
+  } else {
+    cudaStreamCaptureStatus status;
+    const cudaStream_t s = cudaStreamIsCapturing(nullptr, &status) == cudaSuccess ? nullptr : cudaStreamPerThread;
+    cudaGetLastError();
+    for (void* p : all)
+      if (cudaFreeAsync(p, s) != cudaSuccess) failed.push_back(p);
   }
+  if (failed.empty()) return;
+  cudaGetLastError();
   std::lock_guard<std::mutex> lock(g_late_mu);
-  g_late[dev].insert(g_late[dev].end(), all.begin(), all.end());
+  g_late[dev].insert(g_late[dev].end(), failed.begin(), failed.end());
 }
 
 int dalloc_async(void** p, size_t bytes, int64_t* counter, cudaStream_t s) {

@@ -41,22 +41,37 @@ int dalloc_n(T** p, size_t n, int64_t* counter) {
 }
 void dfree(void* p);
 // Stream-ordered allocation on s from the device's default memory pool (which
-// keeps up to 8 GB of freed memory for reuse).  To be released by dfree_idle:
-// unlike that of dalloc's memory, the free of the pool's waits for nothing.
+// keeps up to 8 GB of freed memory for reuse), to be released by dfree_pooled:
+// unlike that of dalloc's memory, cudaFree of the pool's waits for nothing.
 int dalloc_async(void** p, size_t bytes, int64_t* counter, cudaStream_t s);
 template <class T>
 int dalloc_async_n(T** p, size_t n, int64_t* counter, cudaStream_t s) {
   return dalloc_async(reinterpret_cast<void**>(p), n * sizeof(T), counter, s);
 }
-
 // A word each of device and of pinned host memory that live on, so that the
 // chunks of memory they lie in stay mapped: a small solver's arrays and the
-// wait in dfree_idle would otherwise map and unmap a chunk each time (97 us
+// wait in dfree_pooled would otherwise map and unmap a chunk each time (97 us
 // against 3 for an allocation and its free).
 void keep_chunks();
-// Frees arrays of the current device (of either kind, null ones skipped) once
-// the work launched on it so far has finished.
-void dfree_idle(void* const* ptrs, size_t n);
+
+// Whether a handle's arrays have been used on a stream other than the default
+// one.  (A stream's handle is no use later: the caller may have destroyed it.)
+struct StreamUse {
+  mutable std::atomic<bool> other{false};
+  void on(cudaStream_t s) const {
+    if (s != nullptr) other.store(true, std::memory_order_relaxed);
+  }
+};
+// Frees arrays of dalloc_async (null ones skipped): in the default stream's
+// order where all their uses were in it, else once the work launched on the
+// device so far has finished.  (A newly assembled operator per step, 1.03 M
+// rows with block Jacobi and an apply of each: 468 us with the wait, 425
+// without.)  Freed in the default stream, whose next allocation finds the
+// arrays at once; after a cudaFree it looks through all streams that have used
+// the pool, 0.8 us for each.  While a blocking stream is being captured the
+// default stream may not be used: then in the thread's own default stream,
+// which is ordered with it.
+void dfree_pooled(void* const* ptrs, size_t n, const StreamUse& use);
 
 // Number of SMs of the current device (cached per device).
 int sm_count();
@@ -289,6 +304,7 @@ struct Matrix {
   double* stage_in = nullptr;   // host-vector staging
   double* stage_out = nullptr;
   int max_grid = 0;             // partials hold max_grid * 2 doubles
+  StreamUse use;
 };
 
 void matrix_release(Matrix* A);
@@ -345,6 +361,7 @@ struct Precond {
   double* stage_in = nullptr;
   double* stage_out = nullptr;
   int64_t device_bytes = 0;
+  StreamUse use;
 };
 
 void precond_release(Precond* P);
@@ -365,6 +382,7 @@ struct Solver {
   gk_criteria crit{};
   int64_t n = 0;
   int64_t device_bytes = 0;
+  double* vecs = nullptr;  // the vectors, one behind the other:
   double *b = nullptr, *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *z = nullptr;
   double *rh = nullptr, *ph = nullptr, *s = nullptr, *sh = nullptr, *t = nullptr;
   SolverState* st = nullptr;
@@ -391,9 +409,11 @@ struct Solver {
   size_t gr_smem = 0;
   int gr_halo_cap = 0;              // its largest halo
   unsigned long long gr_epoch = 0;  // the next solve's sequence numbers start at gr_epoch << 40
-  ulonglong2* gr_words = nullptr;   // {value, sequence number}: the reductions', the abort word, the vectors'
+  StreamUse use;
   int32_t* gr_halo_n = nullptr;     // halo entries of every CTA
-  int32_t* gr_halo_col = nullptr;   // and their columns
+  void* gr_plan = nullptr;          // one array with the next three
+  ulonglong2* gr_words = nullptr;   // {value, sequence number}: the reductions', the abort word, the vectors'
+  int32_t* gr_halo_col = nullptr;   // the halos' columns
   int32_t* gr_code = nullptr;       // per entry of the matrix, its column's place in the CTA's slice
 };
 

@@ -997,8 +997,7 @@ constexpr size_t kGrSmemMax = 216 * 1024;
 }  // namespace
 
 // cluster: the plan of the 16-CTA form (the caller has checked that the
-// cluster form applies); else of the cooperative grid.  Its arrays come from
-// the pool, like the operator's.
+// cluster form applies); else of the cooperative grid.
 int grid_cg_plan(Solver* S, bool cluster) {
   S->gr_grid = 0;
   if ((S->kind != GK_CG && S->kind != GK_BICGSTAB) || S->pk == PREC_BLOCK) return GK_OK;
@@ -1020,7 +1019,7 @@ int grid_cg_plan(Solver* S, bool cluster) {
   // the CTAs' halos, entries and longest rows, then the lists
   const size_t plan_smem = 8 * static_cast<size_t>((n + 31) / 32);
   GK_TRY(set_smem(gr_halo_kernel, plan_smem));
-  GK_TRY(dalloc_async_n(&S->gr_halo_n, static_cast<size_t>(3 * G), &S->device_bytes, nullptr));
+  GK_TRY(dalloc_n(&S->gr_halo_n, static_cast<size_t>(3 * G), &S->device_bytes));
   gr_halo_kernel<<<G, kGrPlanThreads, plan_smem>>>(S->A->rowptr, S->A->col, static_cast<int>(n), static_cast<int>(R),
                                                    0, S->gr_halo_n, nullptr, nullptr);
   GK_TRY_CUDA(cudaGetLastError());
@@ -1057,9 +1056,13 @@ int grid_cg_plan(Solver* S, bool cluster) {
     return GK_OK;
   }
   const size_t n_words = static_cast<size_t>(2) * kGrCopies * kGrMaxK * G + 1, n_vec = static_cast<size_t>(bi ? 4 : 2) * n;
-  GK_TRY(dalloc_async_n(&S->gr_words, n_words + n_vec, &S->device_bytes, nullptr));
-  GK_TRY(dalloc_async_n(&S->gr_halo_col, static_cast<size_t>(G) * cap, &S->device_bytes, nullptr));
-  GK_TRY(dalloc_async_n(&S->gr_code, static_cast<size_t>(std::max<int64_t>(S->A->nnz, 1)), &S->device_bytes, nullptr));
+  const size_t n_col = static_cast<size_t>(G) * cap, n_code = static_cast<size_t>(S->A->nnz);
+  GK_TRY(dalloc_async(&S->gr_plan, (n_words + n_vec) * sizeof(ulonglong2) + (n_col + n_code) * sizeof(int32_t),
+                      &S->device_bytes, nullptr));
+  S->gr_words = static_cast<ulonglong2*>(S->gr_plan);
+  // (codes on a 16-byte boundary)
+  S->gr_code = reinterpret_cast<int32_t*>(S->gr_words + n_words + n_vec);
+  S->gr_halo_col = S->gr_code + n_code;
   GK_TRY_CUDA(cudaMemset(S->gr_words, 0, (n_words + n_vec) * sizeof(ulonglong2)));
   gr_halo_kernel<<<G, kGrPlanThreads, plan_smem>>>(S->A->rowptr, S->A->col, static_cast<int>(n), static_cast<int>(R),
                                                    static_cast<int>(cap), S->gr_halo_n, S->gr_halo_col, S->gr_code);

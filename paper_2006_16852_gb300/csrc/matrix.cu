@@ -570,10 +570,13 @@ void matrix_release(Matrix* A) {
                   A->ell_val,
                   A->tail_rows, A->tail_rowptr, A->tail_row, A->tail_col, A->tail_val, A->tail_slot,
                   A->tail_sum, A->coo_first, A->coo_last, A->coo_head, A->coo_tail, A->partials, A->counter,
-                  A->err, A->dot_st, A->stage_in, A->stage_out};
+                  A->err};
   // applies are asynchronous, and a failed creation leaves kernels behind:
   // the pool must not hand these arrays out before they have finished
-  dfree_idle(ptrs, sizeof(ptrs) / sizeof(ptrs[0]));
+  dfree_pooled(ptrs, sizeof(ptrs) / sizeof(ptrs[0]), A->use);
+  dfree(A->dot_st);
+  dfree(A->stage_in);
+  dfree(A->stage_out);
   if (prev >= 0) cudaSetDevice(prev);
   delete A;
 }
@@ -607,6 +610,7 @@ extern "C" int gk_matrix_create_csr(int64_t n_rows, int64_t n_cols, int64_t nnz,
   A->n_rows = n_rows;
   A->n_cols = n_cols;
   A->nnz = nnz;
+  A->use.on(s);
   int64_t* bytes = &A->device_bytes;
 
   // ---- library-owned CSR copy, checked and analysed on the way -----------------

@@ -431,8 +431,10 @@ void precond_release(Precond* P) {
   int prev = -1;
   cudaGetDevice(&prev);
   cudaSetDevice(P->device);
-  void* ptrs[] = {P->dinv, P->blocks, P->stage_in, P->stage_out};
-  dfree_idle(ptrs, 4);
+  void* ptrs[] = {P->dinv, P->blocks};
+  dfree_pooled(ptrs, 2, P->use);
+  dfree(P->stage_in);
+  dfree(P->stage_out);
   matrix_release(P->A);
   if (prev >= 0) cudaSetDevice(prev);
   delete P;
@@ -440,6 +442,7 @@ void precond_release(Precond* P) {
 
 int precond_apply_launch(const Precond* P, const double* r, double* z, cudaStream_t s) {
   if (P->n == 0) return GK_OK;
+  P->use.on(s);
   if (P->bs == 1) {
     scalar_apply_kernel<<<grid_for(P->n, 256), 256, 0, s>>>(P->dinv, r, z, P->n);
   } else {
@@ -477,6 +480,8 @@ extern "C" int gk_precond_generate(gk_matrix h, int32_t block_size, void* stream
   P->A = A;
   P->n = A->n_rows;
   P->bs = block_size;
+  A->use.on(s);
+  P->use.on(s);
   int rc = GK_OK;
   do {
     // the error word: 0, or INT_MAX - the smallest failing row or block
@@ -554,6 +559,7 @@ extern "C" int gk_precond_get_blocks(gk_precond h, double* out, int64_t n_out, v
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int rc = GK_OK;
   do {
+    P->use.on(s);
     // the device layout is the exported one: row-major blocks, concatenated
     const double* src = P->bs == 1 ? P->dinv : P->blocks;
     if (cudaMemcpyAsync(out, src, sizeof(double) * total, cudaMemcpyDefault, s) != cudaSuccess) {

@@ -507,12 +507,12 @@ void solver_release(Solver* S) {
   if (S->exec) cudaGraphExecDestroy(S->exec);
   if (S->graph) cudaGraphDestroy(S->graph);
   if (S->cs) cudaStreamDestroy(S->cs);
-  void* const pooled[] = {S->b, S->x, S->r,  S->p, S->q,        S->z,         S->rh,         S->ph,
-                          S->s, S->sh, S->t, S->gr_words, S->gr_halo_n, S->gr_halo_col, S->gr_code};
-  dfree_idle(pooled, sizeof(pooled) / sizeof(pooled[0]));
+  void* const pooled[] = {S->vecs, S->gr_plan};
+  dfree_pooled(pooled, sizeof(pooled) / sizeof(pooled[0]), S->use);
   dfree(S->st);
   dfree(S->partials);
   dfree(S->counter);
+  dfree(S->gr_halo_n);
   if (S->h_st) cudaFreeHost(S->h_st);
   ir_release(S->ir);
   gmres_release(S->gm);
@@ -704,10 +704,14 @@ int build_graph(Solver& S) {
   return GK_OK;
 }
 
-// From the pool, like the operator's arrays: mapped and unmapped for each
-// solver of 65,536 rows, five vectors take 150 us.
-int alloc_vec(double** v, int64_t n, int64_t* bytes) {
-  return dalloc_async_n(v, static_cast<size_t>(std::max<int64_t>(n, 1)), bytes, nullptr);
+// The solver's vectors, in one array of the pool: five of cudaMalloc take a
+// solver of 65,536 rows 150 us to map and unmap, and an allocation of the pool
+// about 1 us for every stream that has used it.
+int alloc_vecs(Solver* S, const std::vector<double**>& vecs) {
+  const size_t ld = static_cast<size_t>((std::max<int64_t>(S->n, 1) + 63) / 64 * 64);  // 512-byte boundaries, as the pool's
+  GK_TRY(dalloc_async_n(&S->vecs, ld * vecs.size(), &S->device_bytes, nullptr));
+  for (size_t i = 0; i < vecs.size(); ++i) *vecs[i] = S->vecs + i * ld;
+  return GK_OK;
 }
 
 }  // namespace
@@ -750,24 +754,15 @@ extern "C" int gk_solver_generate(gk_matrix hA, gk_precond hP, int32_t kind, con
   int rc = GK_OK;
   keep_chunks();
   do {
-    if ((rc = alloc_vec(&S->b, S->n, by)) || (rc = alloc_vec(&S->x, S->n, by)) ||
-        (rc = alloc_vec(&S->r, S->n, by)) || (rc = alloc_vec(&S->p, S->n, by)) ||
-        (rc = alloc_vec(&S->q, S->n, by)))
-      break;
-    if ((kind == GK_CG || kind == GK_FCG) && S->pk != PREC_NONE && (rc = alloc_vec(&S->z, S->n, by))) break;
-    if (kind == GK_CGS) {
-      if ((rc = alloc_vec(&S->rh, S->n, by)) || (rc = alloc_vec(&S->s, S->n, by)) ||
-          (rc = alloc_vec(&S->t, S->n, by)) || (rc = alloc_vec(&S->sh, S->n, by)))
-        break;
-      if (S->pk != PREC_NONE && (rc = alloc_vec(&S->ph, S->n, by))) break;
-    }
-    if (kind == GK_BICGSTAB) {
-      if ((rc = alloc_vec(&S->rh, S->n, by)) || (rc = alloc_vec(&S->s, S->n, by)) ||
-          (rc = alloc_vec(&S->t, S->n, by)))
-        break;
-      if (S->pk != PREC_NONE && ((rc = alloc_vec(&S->ph, S->n, by)) || (rc = alloc_vec(&S->sh, S->n, by))))
-        break;
-    }
+    std::vector<double**> vecs = {&S->b, &S->x, &S->r, &S->p, &S->q};
+    const auto more = [&](std::initializer_list<double**> v) { vecs.insert(vecs.end(), v); };
+    const bool pre = S->pk != PREC_NONE;
+    if ((kind == GK_CG || kind == GK_FCG) && pre) more({&S->z});
+    if (kind == GK_CGS) more({&S->rh, &S->s, &S->t, &S->sh});
+    if (kind == GK_CGS && pre) more({&S->ph});
+    if (kind == GK_BICGSTAB) more({&S->rh, &S->s, &S->t});
+    if (kind == GK_BICGSTAB && pre) more({&S->ph, &S->sh});
+    if ((rc = alloc_vecs(S, vecs))) break;
     if ((rc = dalloc_n(&S->st, 1, by))) break;
     S->grid_vec = vec_grid(*S);
     const int pg = std::max(S->grid_vec, spmv_max_grid(*A));
@@ -815,6 +810,9 @@ extern "C" int gk_solve(gk_solver h, const void* b, void* x, gk_status* status, 
       }
       break;
     }
+    S->use.on(s);
+    S->A->use.on(s);
+    if (S->P) S->P->use.on(s);
     const size_t vb = sizeof(double) * static_cast<size_t>(S->n);
     cudaError_t e = cudaMemcpyAsync(S->b, b, vb, cudaMemcpyDefault, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(S->x, x, vb, cudaMemcpyDefault, s);

@@ -956,6 +956,7 @@ int spmv_max_grid(const Matrix& A) {
 
 int spmv_launch(const Matrix& A, const double* x, const Epi& e, cudaStream_t s) {
   if (A.n_rows == 0) return GK_OK;
+  A.use.on(s);
   switch (A.format) {
     case GK_CSR: {
       SliceArgs b{A.rowptr, A.col, A.val, A.sl_perm, A.sl_off, A.sl_col, A.sl_val, static_cast<int>(A.n_sell),

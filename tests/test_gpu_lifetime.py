@@ -1,6 +1,7 @@
 """Handles destroyed while work that uses them is still running: their arrays
 come from the stream-ordered pool, which hands freed memory out again at
-once, so the destroying call has to wait for the device."""
+once: the destroying call waits for the device, or frees them in the order of
+the default stream where they were used on no other."""
 import threading
 
 import numpy as np
@@ -55,6 +56,40 @@ def test_destroyed_with_an_apply_in_flight(gk, orc, what):
     torch.cuda.synchronize()
     assert np.array_equal(to_np(y), to_np(want))
     del Q
+
+
+@pytest.mark.parametrize("what", ["csr", "csr_merge", "ell", "hyb", "jacobi", "block jacobi"])
+@pytest.mark.parametrize("same", [True, False])
+def test_destroyed_with_an_apply_in_flight_on_the_default_stream(gk, what, same):
+    """As above on the default stream, in whose order the arrays are freed;
+    the next operators are made on it or on another stream."""
+    import torch
+    ny, nx = 300, 401
+    n = ny * nx
+    A, B = (W.varcoef2d(np.exp(0.5 * np.random.default_rng(k).standard_normal(s))) for k, s in
+            ((1, (ny, nx)), (2, (nx, ny))))
+    b_dev = [to_dev(a) for a in B]
+    x = to_dev(W.uniform_vector(n, 3))
+    fmt = what if "jacobi" not in what else "csr"
+    M = _operator(gk, A, fmt)
+    P = gk.Precond(M, 1 if what == "jacobi" else 8) if "jacobi" in what else None
+    want = torch.empty_like(x)
+    gk.precond_apply(P, x, want) if P else gk.apply(M, x, want)
+    y = torch.full_like(x, float("nan"))
+    torch.cuda.synchronize()
+    done = torch.cuda.Event()
+    torch.cuda._sleep(BUSY)
+    gk.precond_apply(P, x, y) if P else gk.apply(M, x, y)
+    done.record()
+    P = None
+    M = None
+    assert not done.query()  # freed in order, without a wait
+    with torch.cuda.stream(torch.cuda.default_stream() if same else torch.cuda.Stream()):
+        others = [gk.Matrix(*b_dev, fmt=fmt) for _ in range(2)]
+        Q = [gk.Precond(o, 8) for o in others]
+    torch.cuda.synchronize()
+    assert np.array_equal(to_np(y), to_np(want))
+    del Q, others
 
 
 def test_destroyed_while_another_thread_captures(gk):
