@@ -377,8 +377,9 @@ GK_API int gk_batch_destroy(gk_batch B);
 typedef struct gk_wsnet_s* gk_wsnet;
 
 /* batch_max: largest batch of the training / forward calls; dilations: 6
- * values in 1..64.  GK_ERR_UNSUPPORTED when a gradient kernel's shared
- * memory (about 4 * (32 W + 96 (W + 2 d)) bytes) exceeds the device's. */
+ * values in 1..64.  The width is limited: GK_ERR_UNSUPPORTED when a layer's
+ * rows (about 4 * (32 W + 96 (W + 2 d)) bytes) exceed the shared memory of a
+ * block, 227 KB. */
 GK_API int gk_wsnet_create(int32_t H, int32_t W, int32_t batch_max, const int32_t* dilations, gk_wsnet* out);
 GK_API int gk_wsnet_num_params(gk_wsnet N, int64_t* n);
 /* params: host or device floats; resets Adam's moments and step count. */

@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kGmresThreads) gm_precond_kernel(GmArgs a) {
 // h_i = V_i . w for every i <= j in one sweep: chunks of 8 vectors (w is
 // re-read per chunk, from L2), each chunk's per-thread sums reduced to one
 // partial per block; the last block to arrive sums the block partials of
-// every i in block order (warp k takes i = k, k + 16, ...: lane l adds
+// every i in block order (warp k takes i = k, k + 8, ...: lane l adds
 // partials l, l + 32, ... into four interleaved sums so that four loads are
 // in flight, then the four sums and one butterfly) and stores this pass's
 // coefficients and H(i, j) (the first pass sets it, the second adds).

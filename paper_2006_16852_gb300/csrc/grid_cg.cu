@@ -72,7 +72,9 @@ constexpr int kGrWarps = kGrThreads / 32;
 constexpr int kGrMaxCtas = 160;          // 5 words per polling lane
 constexpr int kGrMaxRptCg = 8;           // rows per thread: registers of the row's vectors
 constexpr int kGrMaxRptBi = 4;
-constexpr int64_t kGrMinRows = 32769;    // below: the cluster form (CG), the graph form (BiCGSTAB)
+// Below: the cluster form, for BiCGSTAB (whose cluster form ends at 16,384
+// rows) the graph form; the line is CG's, BiCGSTAB's own has not been measured.
+constexpr int64_t kGrMinRows = 32769;
 constexpr int64_t kGrMaxRows = 262144;   // above: the graph form's SpMV kernels win
 constexpr int kGrMaxRowLen = 64;         // one thread per row: no long rows
 constexpr int kGrMaxK = 3;               // values per reduction
@@ -990,9 +992,11 @@ cudaLaunchConfig_t cluster_config(size_t smem, cudaStream_t s, cudaLaunchAttribu
   return cfg;
 }
 
-// Dynamic shared memory a CTA may use (of 227 KB, next to the reductions' 6
-// KB): the vectors must fit, the rows of the matrix are staged if they do.
+// Dynamic shared memory a CTA may use (of 227 KB, next to the 7.7 KB of the
+// reductions and the scalars): the vectors must fit, the rows of the matrix
+// are staged if they do.
 constexpr size_t kGrSmemMax = 216 * 1024;
+static_assert(sizeof(GridRed) + sizeof(GrScalars) + kGrSmemMax <= 227 * 1024, "a CTA's shared memory");
 
 }  // namespace
 

@@ -199,7 +199,9 @@ constexpr int kDeepMinLen = 8;
 // work: 8 % there).
 // Power-law of 10^6 rows: 167.9 -> 141.6 us an apply, 1.08x the gather
 // ceiling (back to back 150.6 -> 139.4, with the fused dot 171.4 -> 155.2);
-// 300,000 rows 80 -> 60 us; 120,000 rows 58 -> 38 us.
+// 300,000 rows 80 -> 60 us; 120,000 rows 58 -> 38 us.  (Within the 32 and 40
+// registers of 8 and 6 blocks per SM the compiler spills 7 to 20 words a
+// thread here, 28 to 80 bytes; the figures are with them.)
 enum SliceKind { SL_PLAIN = 0, SL_DEEP = 1, SL_SPLIT = 2 };
 
 // The line: slices of more than 0.6 times a warp's share of all slots, and at

@@ -1356,7 +1356,7 @@ struct WsNet {
   bool bf_stale = true;
   float* act[kLayers + 1] = {};  // act[0] unused (the caller's input); act[l + 1] = layer l output
   float* dbuf[2] = {};           // data-gradient ping-pong
-  __nv_bfloat16* hbf[3] = {};    // inference: [1], [2] ping-pong activations (layout of tc_act)
+  __nv_bfloat16* hbf[2] = {};    // inference: ping-pong activations (layout of tc_act)
   __nv_bfloat16* wtc = nullptr;  // the 32 -> 32 layers' weights in the tensor-core layout
   int* err = nullptr;            // device-side wait that gave up (kErrTimeout)
   int tc_smem_sm = 0, tc_reserved = 0;  // shared memory per SM and reserved per block
@@ -1380,7 +1380,7 @@ void wsnet_release(WsNet* N) {
   const int prev = current_device();
   cudaSetDevice(N->device);
   void* ptrs[] = {N->p,      N->g,      N->m,        N->v,     N->wflip,   N->pbf,  N->dbuf[0],
-                  N->dbuf[1], N->hbf[0], N->hbf[1],   N->hbf[2], N->partials, N->chunk, N->red,
+                  N->dbuf[1], N->hbf[0], N->hbf[1], N->partials, N->chunk, N->red,
                   N->counter, N->dred,   N->dcounter, N->scal,  N->feat,     N->ax,      N->wtc, N->err};
   for (void* q : ptrs) dfree(q);
   for (int l = 1; l <= kLayers; ++l) dfree(N->act[l]);
@@ -1420,8 +1420,9 @@ int forward_layer(int l, const float* x, const float* w, const float* bias, int 
   return launch_conv<32, 1, CONV_LINEAR>(x, w, bias, B, H, W, dil, y, nullptr, s);
 }
 
-// The documented limit on the width: the shared memory that one row of a
-// layer's two tensors, three input rows with their halo, would take.
+// The documented limit on the width: one row of a layer's two tensors, three
+// input rows with their halo, would fit a block's shared memory.  (No kernel
+// stages whole rows any more.)
 size_t width_limit_bytes(int cin, int cout, int W, int dil) {
   const int co_t = cout >= 4 ? 4 : 1;
   const size_t xsplit = kConvThreads / (cin * (cout / co_t));
@@ -1538,11 +1539,11 @@ int infer_bf16(WsNet& N, int B, const float* x, float* y, cudaStream_t s) {
   // 8 resident blocks per SM: 64 of the 512 tensor-memory columns each
   const int grid1 = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(tiles, 8 * sm_count())));
   conv_first_tc_kernel<<<grid1, kTcFirstThreads, 0, s>>>(x, N.pbf + N.off_w[0], N.pbf + N.off_b[0], B, N.H, N.W,
-                                                         N.dil[0], strip_for(grid1, N.dil[0]), N.hbf[1], N.err);
+                                                         N.dil[0], strip_for(grid1, N.dil[0]), N.hbf[0], N.err);
   GK_TRY_CUDA(cudaGetLastError());
-  const __nv_bfloat16* in = N.hbf[1];
+  const __nv_bfloat16* in = N.hbf[0];
   for (int l = 1; l < kLayers - 1; ++l) {
-    __nv_bfloat16* out = N.hbf[1 + (l & 1)];
+    __nv_bfloat16* out = N.hbf[l & 1];
     // resident blocks per SM: shared memory is the limit (registers, warps
     // and the 512 tensor-memory columns allow 8 blocks of 64 columns), and
     // it depends on the dilation through the staged rows' width
@@ -1603,7 +1604,7 @@ extern "C" int gk_wsnet_create(int32_t H, int32_t W, int32_t batch_max, const in
   GK_TRY_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, N->device));
   for (int l = 0; l < kLayers; ++l)
     if (width_limit_bytes(kCh[l], kCh[l + 1], W, N->dil[l]) > static_cast<size_t>(smem_max))
-      return set_error(GK_ERR_UNSUPPORTED, "gk_wsnet_create: width %d with dilation %d needs too much shared memory",
+      return set_error(GK_ERR_UNSUPPORTED, "gk_wsnet_create: width %d with dilation %d exceeds the limit",
                        W, N->dil[l]);
   int64_t* by = &N->device_bytes;
   const size_t np = static_cast<size_t>(off);
@@ -1614,8 +1615,7 @@ extern "C" int gk_wsnet_create(int32_t H, int32_t W, int32_t batch_max, const in
   for (int l = 1; l <= kLayers; ++l)
     GK_TRY(dalloc_n(&N->act[l], l < kLayers ? big : static_cast<size_t>(batch_max) * img, by));
   for (float** q : {&N->dbuf[0], &N->dbuf[1]}) GK_TRY(dalloc_n(q, big, by));
-  GK_TRY(dalloc_n(&N->hbf[1], big, by));
-  GK_TRY(dalloc_n(&N->hbf[2], big, by));
+  for (__nv_bfloat16** q : {&N->hbf[0], &N->hbf[1]}) GK_TRY(dalloc_n(q, big, by));
   GK_TRY(dalloc_n(&N->wtc, static_cast<size_t>(kTcMidLayers) * kTcPacked, by));
   GK_TRY(dalloc_n(&N->err, 1, by));
   GK_TRY_CUDA(cudaMemset(N->err, 0, sizeof(int)));
