@@ -488,10 +488,13 @@ GK_API int gk_dot_noalloc(int64_t n, const double* x, const double* y, double* r
  * the kernel return, so a stalled wait ends the call with GK_ERR_TIMEOUT (or
  * gk_status.device_error) instead of hanging the GPU.  This call launches one
  * warp that waits, through the same code, on a barrier phase that nothing
- * completes; it returns after the wait has given up (about 2 s at the
- * maximum SM clock) with *err_out = the device error word: 1 when the wait
- * timed out as designed.  The device stays usable afterwards.  Synchronous
- * on stream; allocates and frees 4 bytes of device memory. */
+ * completes, and then a block that waits for a word that nobody writes, as the
+ * one-launch solvers' reductions do; it returns after both waits have given up
+ * (about 2 s each at the maximum SM clock) with *err_out = the device error
+ * word: 1 when the first timed out as designed, and 4 added unless the second
+ * did and ended the block's other waits at once.  The device stays usable
+ * afterwards.  Synchronous on stream; allocates and frees a few KB of device
+ * memory. */
 GK_API int gk_wait_selftest(int32_t* err_out, void* stream);
 
 #ifdef __cplusplus

@@ -438,8 +438,8 @@ def fp64_rate(iters: int = 20000, stream=None) -> float:
 
 
 def wait_selftest(stream=None) -> int:
-    """Runs one bounded device-side wait that nothing satisfies; returns the
-    device error word it leaves (1: the wait gave up, as designed)."""
+    """Runs the bounded device-side waits on what never comes; returns the
+    device error word they leave (1: they gave up, as designed)."""
     err = ctypes.c_int32(-1)
     _check(lib().gk_wait_selftest(ctypes.byref(err), _stream(stream)))
     return err.value

@@ -459,7 +459,8 @@ extern "C" int gk_dot_noalloc(int64_t n, const double* x, const double* y, doubl
 // warp waits, with the same mbar_wait every bulk-copy consumer uses, on an
 // mbarrier phase that nothing completes (one expected arrival, none made, no
 // copy issued).  The wait gives up at its clock limit, sets kErrTimeout in
-// the error word and the kernel returns, so the context stays usable.
+// the error word and the kernel returns, so the context stays usable.  Then
+// the same for the polled words of the one-launch solvers (grid_cg.cu).
 // ---------------------------------------------------------------------------
 namespace gk {
 
@@ -491,7 +492,9 @@ extern "C" int gk_wait_selftest(int32_t* err_out, void* stream) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(d);
   if (e != cudaSuccess) return cuda_error(e, "gk_wait_selftest");
-  *err_out = h;
+  bool polled = false;
+  GK_TRY(grid_wait_selftest(&polled, s));
+  *err_out = polled ? h : h | 4;
   return GK_OK;
 }
 

@@ -436,6 +436,8 @@ int cluster_cg_solve(Solver* S, cudaStream_t s);
 // shared memory (gr_grid > 0 after the plan).
 int grid_cg_plan(Solver* S, bool cluster);
 int grid_cg_solve(Solver* S, bool cluster, cudaStream_t s);
+// Whether a polled word that never comes ends its wait, and the others', as designed.
+int grid_wait_selftest(bool* ok, cudaStream_t s);
 
 // Restarted GMRES (gmres.cu).
 int gmres_generate(Solver* S);

@@ -939,6 +939,31 @@ __global__ void __launch_bounds__(kGrPlanThreads) gr_halo_kernel(const int32_t* 
   }
 }
 
+// The waits' failure path (gk_wait_selftest): thread 0 polls a word that
+// nobody writes, through the halo's fetch, until it gives up; then every
+// thread's wait has to end at the abort word.  *result: 0 if all of it went
+// as designed.
+__global__ void __launch_bounds__(kGrThreads) grid_wait_selftest_kernel(GridArgs a, int* result) {
+  __shared__ GridRed red;
+  __shared__ double dst[4 * kGrThreads];
+  if (threadIdx.x == 0) red.ok = 1;
+  __syncthreads();
+  fetch_halo(a, red, a.words, a.seq0, a.halo_col, 1, dst, 0);
+  __syncthreads();
+  const bool first = red.ok == 0 && *a.abort_ == 1u && (a.st->err & kErrTimeout) != 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    red.ok = 1;
+    a.st->err = 0;
+  }
+  __syncthreads();
+  const long long t0 = clock64();
+  fetch_halo(a, red, a.words, a.seq0, a.halo_col, 4 * kGrThreads, dst, 0);
+  const bool soon = clock64() - t0 < kMaxWaitCycles / 8;
+  const bool all_soon = __syncthreads_and(soon) != 0;
+  if (threadIdx.x == 0) *result = first && all_soon && red.ok == 0 && a.st->err == 0 ? 0 : 1;
+}
+
 using GrKernel = void (*)(GridArgs);
 
 template <int PK, int SRC, bool CLUSTER>
@@ -999,6 +1024,37 @@ constexpr size_t kGrSmemMax = 216 * 1024;
 static_assert(sizeof(GridRed) + sizeof(GrScalars) + kGrSmemMax <= 227 * 1024, "a CTA's shared memory");
 
 }  // namespace
+
+int grid_wait_selftest(bool* ok, cudaStream_t s) {
+  // one array: the state, the abort word, the result, one word, 4 * 256 halo columns (all of them 0)
+  struct Scratch {
+    SolverState st;
+    unsigned int abort_;
+    int result;
+    alignas(16) ulonglong2 word;
+    int32_t cols[4 * kGrThreads];
+  };
+  Scratch* d = nullptr;
+  GK_TRY_CUDA(cudaMalloc(&d, sizeof(Scratch)));
+  GridArgs a = {};
+  a.st = &d->st;
+  a.abort_ = &d->abort_;
+  a.words = &d->word;
+  a.halo_col = d->cols;
+  a.seq0 = 1ull << 40;
+  int result = 1;
+  cudaError_t e = cudaMemsetAsync(d, 0, sizeof(Scratch), s);
+  if (e == cudaSuccess) {
+    grid_wait_selftest_kernel<<<1, kGrThreads, 0, s>>>(a, &d->result);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&result, &d->result, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFree(d);
+  if (e != cudaSuccess) return cuda_error(e, "gk_wait_selftest");
+  *ok = result == 0;
+  return GK_OK;
+}
 
 // cluster: the plan of the 16-CTA form (the caller has checked that the
 // cluster form applies); else of the cooperative grid.
