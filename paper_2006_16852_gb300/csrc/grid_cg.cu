@@ -420,9 +420,16 @@ struct GridRows {
 // (scale), and a norm's square root is taken only where the criteria may
 // hold: rr > tol2 implies ||r|| > tol.  An inverse that is no normal number
 // (the divisor below 5.6e-309 or above 4.5e307, as with a right-hand side
-// scaled near 1e-150 or 1e150) is not used: beta is then the quotient itself.
+// scaled near 1e-150 or 1e150) is not used: beta is then the quotient itself,
+// by a call, so that its divisions stay out of the way (inlined, and with the
+// inverse's factors checked one by one, BiCGSTAB on 100 x 110 took 2,345 us,
+// 2,334 so, 2,327 without any check).
 __device__ __forceinline__ bool gr_normal(double v) {
   return ((static_cast<unsigned int>(__double2hiint(v)) >> 20) & 0x7ffu) - 1u < 0x7feu;
+}
+
+__device__ __noinline__ double gr_slow_beta(double rho, double prev, double alpha, double omega) {
+  return (rho / prev) * (alpha / omega);
 }
 
 struct GrScalars {
@@ -617,7 +624,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) cg_grid_kernel(GridArgs a) {
               [&](int warp, int lane, const double* tt) {
                 if (lane != 0) return;
                 if (warp == 0) {
-                  sc.beta = gr_normal(sc.scale) ? tt[0] * sc.scale : tt[0] / sc.rho;
+                  sc.beta = gr_normal(sc.scale) ? tt[0] * sc.scale : gr_slow_beta(tt[0], sc.rho, 1.0, 1.0);
                   sc.rho = tt[0];
                 } else {
                   sc.iter += 1;
@@ -687,8 +694,11 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
     if (!isfinite(rho)) sc.stop = GK_STOP_NAN;
     else if (rho == 0.0) sc.stop = GK_STOP_BREAKDOWN;
     else {
-      // scale = (alpha / omega) / the previous rho
-      sc.beta = gr_normal(sc.scale) ? rho * sc.scale : (rho / sc.rho) * (sc.alpha / sc.omega);
+      // scale = (alpha / omega) / the previous rho = (1 / r^.v) (t.t / s.t).
+      // The first factor loses 4 bits at most where it is subnormal, the
+      // second more where omega is that large.
+      const bool usable = gr_normal(sc.scale) && fabs(sc.omega) < 0x1p1000;
+      sc.beta = usable ? rho * sc.scale : gr_slow_beta(rho, sc.rho, sc.alpha, sc.omega);
       sc.rho = rho;
     }
   };
@@ -752,7 +762,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
                   const double rhv = tt[0];
                   const double q = (lane == 0 ? sc.rho : 1.0) / rhv;
                   if (lane == 1) {
-                    sc.scale = gr_normal(q) ? q : nan("");
+                    sc.scale = q;
                     return;
                   }
                   sc.spmvs += 1;
@@ -792,7 +802,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) bicg_grid_kernel(GridArgs a) {
                 // (alpha / omega) / rho = (1 / r^.v) (t.t / s.t)
                 const double q = tt[lane == 0 ? 0 : 2] / tt[lane == 0 ? 2 : 0];
                 if (lane == 1) {
-                  sc.scale = gr_normal(q) ? sc.scale * q : nan("");
+                  sc.scale *= q;
                   return;
                 }
                 if (!isfinite(tt[2]) || !isfinite(tt[0])) sc.om_stop = GK_STOP_NAN;
