@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kDotThreads) gm_dots_kernel(GmArgs a) {
     const double* Vc = a.V + static_cast<int64_t>(c0) * a.ldv;
     const int stride = gridDim.x * kDotThreads;
     int r = blockIdx.x * kDotThreads + threadIdx.x;
-    for (; r + (U - 1) * stride < a.n; r += U * stride) {
+    for (; r < a.n - (U - 1) * stride; r += U * stride) {  // (a sum on the left could overflow)
       double wr[U], v[U][N];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
