@@ -871,7 +871,7 @@ extern "C" int gk_solve(gk_solver h, const void* b, void* x, gk_status* status, 
         if (S->crit.time_limit_s > 0 &&
             std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count() >
                 S->crit.time_limit_s) {
-          int tstop = GK_STOP_TIME;
+          static const int tstop = GK_STOP_TIME;  // outlives the copy
           cudaMemcpyAsync(&S->st->stop, &tstop, sizeof(int), cudaMemcpyHostToDevice, s);
           break;
         }
