@@ -608,7 +608,7 @@ def run_batched(dev, reps=3, n_sys=10000, only=None, tune=True, plain=True):
             fl = batch_fp64_flops(kind, True, st["iters"].astype(np.float64), nnz_s, n_s)
             f["fp64_tflops"] = round(fl / (ms * 1e-3) / 1e12, 4)
         forms[name] = f
-        launches[name] = sum(1 for c in chosen if c)
+        launches[name] = 1 + sum(1 for c in chosen if c)  # the vectors' addresses, and a kernel per class
     out = {"workload": BATCH_WORKLOAD, "n_sys": n_sys, "rows": n, "nnz": int(A[1].size),
            "timing": "CUDA events around each gk_batch_solve graph launch, median of %d, inputs resident" % reps,
            "forms": forms, "gpu_launches_per_solve": launches}
