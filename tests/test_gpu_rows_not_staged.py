@@ -55,10 +55,11 @@ def test_against_graph_form(gk, orc, kind, prec, n, reach):
     assert abs(out[0].iters - out[1].iters) <= slack, (out[0].iters, out[1].iters)
 
 
-def test_long_rows_are_not_slower_than_across_the_cluster(gk):
-    """61 diagonals on 16,000 rows: the kernels that read the direction vector
-    across the cluster took 66.5 us an iteration, this form with one entry per
-    load 77 us, with 16-byte loads 43."""
+def test_long_rows_against_the_graph_form(gk):
+    """61 diagonals on 16,000 rows: an iteration took the kernels that read the
+    direction vector across the cluster 2.7 times as long as the graph form,
+    this form 3.4 times with one entry per load and 1.9 times with 16-byte
+    loads."""
     import torch
     n, half = 16000, 30
     i = np.arange(n)
@@ -68,14 +69,17 @@ def test_long_rows_are_not_slower_than_across_the_cluster(gk):
         c += [i[:-d], i[d:]]
     r, c = np.concatenate(r), np.concatenate(c)
     A = W._coo_to_csr(n, r, c, np.where(r == c, 2.0 * half + 1.0, -1.0))
-    S = _solver(gk, A, "cg", 1, max_iters=100, reduction_factor=1e-300)
     b = to_dev(W.uniform_vector(n, 12))
-    best = 1.0
-    for _ in range(5):
-        x = torch.zeros_like(b)
-        torch.cuda.synchronize()
-        t0 = time.perf_counter()
-        st = gk.solve(S, b, x)
-        best = min(best, time.perf_counter() - t0)
-    assert st.form == gk.FORM_CLUSTER and st.iters == 100
-    assert best <= 100 * 60e-6, best
+    best = []
+    for check_every, form in ((0, gk.FORM_CLUSTER), (-1, gk.FORM_GRAPH)):
+        S = _solver(gk, A, "cg", 1, max_iters=100, reduction_factor=1e-300, check_every=check_every)
+        took = []
+        for _ in range(7):
+            x = torch.zeros_like(b)
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            st = gk.solve(S, b, x)
+            took.append(time.perf_counter() - t0)
+        assert st.form == form and st.iters == 100
+        best.append(min(took))
+    assert best[0] <= 2.4 * best[1], best

@@ -12,8 +12,8 @@ from helpers import to_dev, to_np
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("kind", ["cg", "bicgstab", "fcg", "gmres"])
-@pytest.mark.parametrize("side", [8, 64, 128])
+@pytest.mark.parametrize("kind,side", [(k, s) for k in ("cg", "bicgstab", "fcg", "gmres") for s in (8, 64, 128)
+                                       if (k, s) != ("gmres", 128)])  # whose basis is too large for a shared chunk
 def test_generation_of_small_solvers(gk, kind, side):
     """A solver of a small system was made and destroyed in 35 to 60 us while
     the operator's arrays kept its chunk of memory mapped, in 500 to 600 where
